@@ -13,7 +13,11 @@
  *     A Z[:, j] = i * lambda[j] * Z[:, j],   Z^H Z = I.
  * conj(Z[:, j]) is the eigenvector of -i*lambda[j].
  *
- * Route (all on the device, Algorithm 1 in its two-step form, Sec. 2.1/2.3.2):
+ * Route (all on the device, Algorithm 1): a direct reduction to tridiagonal
+ * form (one Householder reflector a column, A <- A + v w^T - w v^T, and the
+ * back transformation by those reflectors alone) where it is the faster one,
+ * which is up to n of about 4000 to 8000 in the FP64 form and the refined
+ * mode; above that, and in the split modes, the two-step form (Sec. 2.1/2.3.2):
  *   full-to-band (blocked Householder panels, compact WY Q = I - V T V^T,
  *   Eq. 7; skew trailing update A <- A + V W^T - W V^T, Eqs. 8-10 with
  *   U1 = -U2), band-to-tridiagonal bulge chase (Sec. 2.3.2, skew SYR2/SYMV),
@@ -119,7 +123,9 @@ typedef struct {
 #define SKEW_TRIDIAG_AUTO 0
 #define SKEW_TRIDIAG_FULL 1
 
-/* skew_opts.qtrd: SKEW_QTRD_AUTO (0) takes the mode's choice (FP64 in the FP64
+/* skew_opts.qtrd: arithmetic of the two-step route's Q_trd.  Any value but
+ * AUTO keeps the two-step route at every order (except SKEW_QTRD_DF where it is
+ * the refined mode's own choice).  SKEW_QTRD_AUTO (0) takes the mode's choice (FP64 in the FP64
  * form; FP32 SIMT when the mixed modes refine; double-float when the refined
  * mode cannot refine (nev < n/2, odd n) and FP64 in the split modes then);
  * the others force FP32 SIMT, FP64 SIMT, the tensor-core form (compact WY

@@ -338,22 +338,24 @@ size_t qband_ws(int n, int b, int k) {
 }
 
 int apply_qband(cudaStream_t st, int n, int b, const double* W, int ldw, const double* Tfac, double* Z, int ldz,
-                int k, void* ws, size_t ws_bytes) {
-    const int P = num_panels(n, b);
+                int k, void* ws, size_t ws_bytes, bool direct) {
+    const int P = direct ? onestep_vcols(n) / b : num_panels(n, b);
     if (P == 0 || k <= 0) return 0;
     Carve cv(ws, ws_bytes);
     QbandWs w = carve_qband(cv, n, b, k);
     if (!cv.ok) return SKEW_ERR_WORKSPACE;
     for (int p = P - 1; p >= 0; p--) {
-        const int o = (p + 1) * b, m = n - o;
+        const int o = direct ? p * b + 1 : (p + 1) * b, m = n - o;
         const double* Tp = Tfac + (size_t)p * b * b;
         double* Zo = Z + o;
         KtScope kt(st, KT_GEMM_F64);
-        if (panel_v(st, n, b, p, W, ldw, w.V, n) != cudaSuccess) return SKEW_ERR_CUDA;
-        if (gemm(st, true, false, b, k, m, 1.0, w.V, n, Zo, ldz, 0.0, w.Y, b, 0, w.part, w.part_n) != cudaSuccess)
+        const double* V = direct ? W + (size_t)p * b * ldw + o : w.V;
+        const int ldv = direct ? ldw : n;
+        if (!direct && panel_v(st, n, b, p, W, ldw, w.V, n) != cudaSuccess) return SKEW_ERR_CUDA;
+        if (gemm(st, true, false, b, k, m, 1.0, V, ldv, Zo, ldz, 0.0, w.Y, b, 0, w.part, w.part_n) != cudaSuccess)
             return SKEW_ERR_CUDA;
         if (gemm(st, false, false, b, k, b, 1.0, Tp, b, w.Y, b, 0.0, w.Y2, b) != cudaSuccess) return SKEW_ERR_CUDA;
-        if (gemm(st, false, false, m, k, b, -1.0, w.V, n, w.Y2, b, 1.0, Zo, ldz) != cudaSuccess) return SKEW_ERR_CUDA;
+        if (gemm(st, false, false, m, k, b, -1.0, V, ldv, w.Y2, b, 1.0, Zo, ldz) != cudaSuccess) return SKEW_ERR_CUDA;
     }
     return 0;
 }
@@ -440,8 +442,9 @@ __global__ void tgroup_init_kernel(int g, int b, const double* __restrict__ Tp, 
 }  // namespace
 
 int apply_qband_mixed(cudaStream_t st, int n, int b, const double* W, int ldw, const double* Tfac, double* Z, int ldz,
-                      int k, void* ws, size_t ws_bytes, int* status, int planes, int slices) {
-    const int P = num_panels(n, b);
+                      int k, void* ws, size_t ws_bytes, int* status, int planes, int slices, bool direct) {
+    const int P = direct ? onestep_vcols(n) / b : num_panels(n, b);
+    if (direct && planes != REDUCE_F64ACC) return SKEW_ERR_UNSUPPORTED;
     if (P == 0 || k <= 0) return 0;
     const bool acc = planes == REDUCE_F64ACC;
     Carve cv(ws, ws_bytes);
@@ -470,14 +473,16 @@ int apply_qband_mixed(cudaStream_t st, int n, int b, const double* W, int ldw, c
     }
     for (int pe = P - 1; pe >= 0; pe -= QG) {
         const int p0 = pe - QG + 1 > 0 ? pe - QG + 1 : 0, g = pe - p0 + 1, gb = g * b;
-        const int o = (p0 + 1) * b, m = n - o;
+        const int o = direct ? p0 * b + 1 : (p0 + 1) * b, m = n - o;
         double* Zo = Z + o;
+        // V of the group (m x gb, ld n): panel p0 + j starts at row j b
+        const double* V = direct ? W + (size_t)p0 * b * ldw + o : q.V;
         {
             KtScope kt(st, KT_GEMM_F64);  // V, T and V T of the group
-            // V of the group (m x gb, ld n): panel p0 + j starts at row j b
-            if (cudaMemsetAsync(V, 0, sizeof(double) * (size_t)n * gb, st) != cudaSuccess) return SKEW_ERR_CUDA;
-            for (int j = 0; j < g; j++)
-                if (panel_v(st, n, b, p0 + j, W, ldw, V + (size_t)j * b * n + (size_t)j * b, n) != cudaSuccess)
+            if (!direct && cudaMemsetAsync(q.V, 0, sizeof(double) * (size_t)n * gb, st) != cudaSuccess)
+                return SKEW_ERR_CUDA;
+            for (int j = 0; j < g && !direct; j++)
+                if (panel_v(st, n, b, p0 + j, W, ldw, q.V + (size_t)j * b * n + (size_t)j * b, n) != cudaSuccess)
                     return SKEW_ERR_CUDA;
             // T of the group
             tgroup_init_kernel<<<(gb * gb + 255) / 256, 256, 0, st>>>(g, b, Tfac + (size_t)p0 * b * b, Tg);

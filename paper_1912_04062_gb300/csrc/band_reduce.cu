@@ -172,6 +172,9 @@ __global__ void __launch_bounds__(TF_THREADS) tfactor_kernel(int nb, const doubl
     double* Ts = sh;             // nb x nb, ld nb + 1
     double* Gs = sh + nb * ld;   // nb x nb, ld nb + 1
     const int t = threadIdx.x;
+    tau += (size_t)blockIdx.x * nb;
+    Gm += (size_t)blockIdx.x * nb * nb;
+    T += (size_t)blockIdx.x * nb * nb;
     for (int e = t; e < nb * nb; e += blockDim.x) {
         const int r = e % nb, c = e / nb;
         Ts[c * ld + r] = 0.0;
@@ -380,6 +383,16 @@ size_t band_reduce_ws(int n, int b, int planes) {
     carve_reduce(cv, n, b, planes == REDUCE_F64ACC);
     if (planes) cv.take<char>(mixed_gemm_ws(n, b, planes));
     return cv.off + 256;
+}
+
+cudaError_t tfactor_panels(cudaStream_t st, int panels, const double* tau, const double* G, double* T) {
+    constexpr int b = 64;
+    if (const cudaError_t e = cudaFuncSetAttribute(tfactor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)tfactor_smem(b)))
+        return e;
+    tfactor_kernel<<<panels, TF_THREADS, tfactor_smem(b), st>>>(b, tau, G, T);
+    count_launch();
+    return cudaGetLastError();
 }
 
 cudaError_t panel_v(cudaStream_t st, int n, int b, int p, const double* W, int ldw, double* V, int ldv) {

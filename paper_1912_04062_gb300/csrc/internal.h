@@ -56,6 +56,33 @@ cudaError_t panel_v(cudaStream_t st, int n, int b, int p, const double* W, int l
                     double* V, int ldv);
 int num_panels(int n, int b);
 
+// T (64 x 64) of each of `panels` panels of 64 reflectors from their Gram
+// matrices (64 x 64 each) and taus (64 each).
+cudaError_t tfactor_panels(cudaStream_t st, int panels, const double* tau, const double* G, double* T);
+
+// ---- onestep.cu (direct tridiagonalisation, FP64) ---------------------------
+// Largest order it takes.
+int onestep_max();
+size_t onestep_ws(int n);
+// Columns of V (and entries of tau): n - 2 rounded up to whole panels of 64.
+int onestep_vcols(int n);
+// Full skew matrix by rows (F[i * n + j]) from the strict lower triangle of A.
+cudaError_t onestep_full(cudaStream_t st, int n, const double* A, int lda, double* F, int check, int* status);
+// F (overwritten) -> alpha (T[c, c + 1], n - 1), V (n x onestep_vcols, ld n:
+// column k is reflector k, zero above row k + 1, one there) and tau.  spin_cap
+// as in band_reduce.
+int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, double* alpha, void* ws,
+                   size_t ws_bytes, int* d_status, unsigned spin_cap);
+// FP64 Z = H_0 H_1 ... H_{n-3} D Q from the interleaved tridiagonal vectors Qi
+// (Qi[i * nev + k]), for the sizes of onestep_wy_fits.
+bool onestep_wy_fits(int n, int nev);
+size_t onestep_back_ws(int n);
+int onestep_back(cudaStream_t st, int n, int nev, const double* V, const double* tau, const double* Qi, double* Zre,
+                 double* Zim, int ldz, void* ws, size_t ws_bytes);
+// T factors of the panels (64 columns of V from column 64 p on), 64 x 64 each.
+int onestep_tfactors(cudaStream_t st, int n, const double* V, const double* tau, double* Tfac, void* ws,
+                     size_t ws_bytes);
+
 // ---- chase.cu ---------------------------------------------------------------
 int chase_steps(int n, int b);
 size_t chase_ws(int n, int b);
@@ -108,10 +135,12 @@ int apply_qtrd_tc(cudaStream_t st, int n, const float* V32, const float* tau32, 
                   void* ws, size_t ws_bytes, int* status);
 size_t qband_ws(int n, int b, int k);
 size_t qband_mixed_ws(int n, int b, int k, int planes);
+// direct: W holds the reflectors of onestep_reduce (explicit columns; panel p
+// starts at row p b + 1 instead of (p + 1) b).
 int apply_qband_mixed(cudaStream_t st, int n, int b, const double* W, int ldw, const double* Tfac, double* Z, int ldz,
-                      int k, void* ws, size_t ws_bytes, int* status, int planes, int slices = 8);
+                      int k, void* ws, size_t ws_bytes, int* status, int planes, int slices = 8, bool direct = false);
 int apply_qband(cudaStream_t st, int n, int b, const double* W, int ldw,
-                const double* Tfac, double* Z, int ldz, int k, void* ws, size_t ws_bytes);
+                const double* Tfac, double* Z, int ldz, int k, void* ws, size_t ws_bytes, bool direct = false);
 
 // ---- umma_gemm.cu (tcgen05 BF16x3) ------------------------------------------
 // C = alpha * split3(A) split3(B)^T + beta * C (FP64 C, column-major, ldc) with

@@ -1,0 +1,677 @@
+// onestep.cu -- one-step Householder tridiagonalisation of a skew-symmetric
+// matrix (the direct form of Sec. 2.3.1: A -> T without the band in between)
+// over the whole GPU, and the FP64 back-transformation by its reflectors.
+//
+// Why one step: the FP64 pipe of this part does 1.68 FMA per clock and SM
+// (measured), so even a matrix-vector product is bound by the arithmetic and
+// not by memory (one element read per 3 FMAs needs 2.8 TB/s over 152 SMs).
+// The two-step route's advantage, products instead of matrix-vector work, is
+// therefore worth nothing in FP64, while its bulge chase (a chain of 2 n
+// dependent tasks) and its second back-transformation (another 4 n^2 nev flops)
+// remain.  Per column c the kernel needs ONE exchange between the CTAs:
+//
+//   every CTA owns the rows i = g (mod G) of the full skew matrix (shared
+//   memory, the rest in L2/HBM) and keeps the current reflector u and
+//   p = A u whole in shared memory;
+//   1. gather (q_j, a_j), j > c: q = A x of the previous reflector's
+//      unscaled column x and a = column c before its rank-2 update.  With
+//      u = x - beta e_0:  A u = q - beta a, so the product could be formed
+//      before beta was known and the norm, sqrt and division are off the
+//      critical path;
+//   2. every CTA forms p, the updated column x = a + sigma (u p_c - p u_c) and, later,
+//      its norm redundantly (same order everywhere: same bits);
+//   3. one pass over the own rows applies A += u w^T - w u^T (Eqs. 2-6 with
+//      u1 = -u2) and multiplies the result by x; the sums and the next column's
+//      elements are published.
+//
+#include <algorithm>
+#include <cfloat>
+
+#include "common.cuh"
+#include "internal.h"
+
+namespace sk {
+namespace {
+
+constexpr int OT = 256;     // threads of the reduction kernel
+constexpr int OW = OT / 32;
+constexpr int OMAXR = 64;   // rows of one CTA at most (n <= 64 G)
+
+struct OsArgs {
+    int n;
+    double* F;     // full skew matrix by rows, F[i * n + j]; rows that are not in shared memory are updated here
+    double* V;     // reflectors by columns (ld n), zeroed by the caller: v[k + 1] = 1
+    double* tau;   // n entries
+    double* alpha; // T[k, k + 1]
+    double2* qa;   // 2 n: (q, a), double-buffered
+    unsigned* ctr; // arrivals (zeroed by the caller)
+    int* status;
+    unsigned cap;
+    int srows;     // own rows kept in shared memory (the last ones: they live longest)
+};
+
+// Totals over the warp of N values per lane by exchanging halves: 5 levels,
+// about N additions instead of 5 N.  Afterwards a[0 .. cnt) of a lane are the
+// totals of the values first .. first + cnt - 1.
+template <int N>
+struct WarpSums {
+    static constexpr int H1 = (N + 1) / 2, H2 = (H1 + 1) / 2, H3 = (H2 + 1) / 2, H4 = (H3 + 1) / 2,
+                         H5 = (H4 + 1) / 2;
+    int first = 0, cnt = N;
+    template <int L, int H, int B>
+    SK_DEV void level(double (&a)[N], int lane) {
+        const bool up = lane & B;
+#pragma unroll
+        for (int i = 0; i < H; i++) {
+            const double hi = (i + H < L) ? a[i + H < N ? i + H : 0] : 0.0;
+            const double keep = up ? hi : a[i], send = up ? a[i] : hi;
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, B);
+        }
+        first += up ? H : 0;
+        cnt = up ? max(cnt - H, 0) : min(cnt, H);
+    }
+    SK_DEV void run(double (&a)[N], int lane) {
+        level<N, H1, 16>(a, lane);
+        level<H1, H2, 8>(a, lane);
+        level<H2, H3, 4>(a, lane);
+        level<H3, H4, 2>(a, lane);
+        level<H4, H5, 1>(a, lane);
+    }
+};
+
+// The rank-2 update of RC own rows (base, base + stride, ...; matrix rows i0,
+// i0 + G, ...) and their products with x, columns ja + 32 (warp + 4 t) + lane.
+// The row sums of this warp go to part[row * OCW].  GLB: rows in global
+// memory, the next step's elements are loaded ahead.
+constexpr int OCW = OW;  // warps of the pass
+
+template <int RC, bool GLB>
+SK_DEV void os_rows(double* base, size_t stride, int i0, int G, int n, int k, int ja, double sigma, const double* u,
+                    const double* p, const double* x, int warp, int lane, double* part) {
+    double ui[RC], pi[RC], acc[RC];
+#pragma unroll
+    for (int r = 0; r < RC; r++) {
+        ui[r] = sigma * u[i0 + r * G];
+        pi[r] = -sigma * p[i0 + r * G];
+        acc[r] = 0.0;
+    }
+    auto step = [&](int j, const double (&in)[RC]) {
+        const double uj = u[j], pj = p[j], xj = (j > k) ? x[j] : 0.0;
+        double a[RC];
+#pragma unroll
+        for (int r = 0; r < RC; r++) a[r] = fma(ui[r], pj, in[r]);
+#pragma unroll
+        for (int r = 0; r < RC; r++) {
+            a[r] = fma(pi[r], uj, a[r]);
+            if (j == i0 + r * G) a[r] = 0.0;
+            base[r * stride + j] = a[r];
+        }
+#pragma unroll
+        for (int r = 0; r < RC; r++) acc[r] = fma(a[r], xj, acc[r]);
+    };
+    int j = ja + 32 * warp + lane;
+    if (GLB) {
+        double nx[RC];
+#pragma unroll
+        for (int r = 0; r < RC; r++) nx[r] = j < n ? base[r * stride + j] : 0.0;
+#pragma unroll 1
+        for (; j < n; j += 32 * OCW) {
+            const int jn = j + 32 * OCW;
+            double in[RC];
+#pragma unroll
+            for (int r = 0; r < RC; r++) {
+                in[r] = nx[r];
+                nx[r] = jn < n ? base[r * stride + jn] : 0.0;
+            }
+            step(j, in);
+        }
+    } else {
+#pragma unroll 1
+        for (; j < n; j += 32 * OCW) {
+            double in[RC];
+#pragma unroll
+            for (int r = 0; r < RC; r++) in[r] = base[r * stride + j];
+            step(j, in);
+        }
+    }
+    WarpSums<RC> ws;
+    ws.run(acc, lane);
+#pragma unroll
+    for (int i = 0; i < WarpSums<RC>::H5; i++)
+        if (i < ws.cnt) part[(ws.first + i) * OCW] = acc[i];
+}
+
+template <bool GLB>
+SK_DEV void os_rows_any(int cnt, double* base, size_t stride, int i0, int G, int n, int k, int ja, double sigma,
+                        const double* u, const double* p, const double* x, int warp, int lane, double* part) {
+    while (cnt > 0) {
+        const int c = min(cnt, 8);
+        switch (c) {
+        case 1: os_rows<1, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
+        case 2: os_rows<2, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
+        case 3: os_rows<3, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
+        case 4: os_rows<4, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
+        case 5: os_rows<5, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
+        case 6: os_rows<6, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
+        case 7: os_rows<7, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
+        default: os_rows<8, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part);
+        }
+        cnt -= c;
+        base += (size_t)c * stride;
+        i0 += c * G;
+        part += c * OCW;
+    }
+}
+
+__global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
+    extern __shared__ __align__(16) double os_sm[];
+    __shared__ double s_part[OMAXR][OCW];
+    __shared__ double s_red[4];
+    __shared__ double s_sc[4];  // beta, sigma, 1 / u_0, u_0
+    __shared__ int s_ok;
+    const int n = o.n, G = gridDim.x, g = blockIdx.x;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int ldn = n | 1;
+    double* u = os_sm;           // u of the pending update (indices k ..)
+    double* p = u + ldn;         // A u of it
+    double* x = p + ldn;         // the column being eliminated
+    double* rows = x + ldn;
+    const int Rt = (n - 1 - g) / G + 1;              // own rows: g, g + G, ...
+    const int rs0 = Rt > o.srows ? Rt - o.srows : 0; // the first one in shared memory
+    const int ilast = g + (Rt - 1) * G;
+    for (int r = rs0; r < Rt; r++)
+        for (int j = t; j < n; j += OT) rows[(size_t)(r - rs0) * ldn + j] = o.F[(size_t)(g + r * G) * n + j];
+    unsigned target = 0;
+    double beta = 0.0, sigma = 0.0;
+    for (int k = 0; k + 1 < n; k++) {
+        if (ilast < k + 1) return;  // no rows left: the others do not count on this CTA any more
+        // ---- 1. gather; p of the previous reflector, the updated column x
+        const double2* qa = o.qa + (size_t)(k & 1) * n;
+        if (k == 0) {
+            // column 0 of A, nothing pending: element (j, 0) = -element (0, j)
+            for (int j = t; j < n; j += OT) {
+                x[j] = -o.F[j];
+                u[j] = 0.0;
+                p[j] = 0.0;
+            }
+        } else {
+            const double2 qk = __ldcg(qa + k);
+            const double uk = -sigma * u[k], pk = sigma * fma(-beta, qk.y, qk.x);
+#pragma unroll 4
+            for (int j = k + 1 + t; j < n; j += OT) {
+                const double2 e = __ldcg(qa + j);
+                const double pj = fma(-beta, e.y, e.x);
+                p[j] = pj;
+                x[j] = fma(u[j], pk, fma(pj, uk, e.y));
+            }
+        }
+        __syncthreads();
+        if (k == n - 2) {
+            // T[n-1, n-2] = x_{n-1}; this CTA owns the last row
+            if (t == 0) o.alpha[k] = -x[n - 1];
+            return;
+        }
+        // ---- 2. update the own rows i > k and multiply by x
+        const int rf = (k + 1 > g) ? (k + 1 - g + G - 1) / G : 0;  // first own row below k
+        const int R = Rt - rf;
+        const int ja = (k + 1) & ~3;
+        const int rg = max(rs0, rf) - rf;  // rows of global memory
+        if (rg > 0)
+            os_rows_any<true>(rg, o.F + (size_t)(g + rf * G) * n, (size_t)G * n, g + rf * G, G, n, k, ja, sigma, u, p,
+                              x, warp, lane, &s_part[0][warp]);
+        os_rows_any<false>(R - rg, rows + (size_t)(rf + rg - rs0) * ldn, ldn, g + (rf + rg) * G, G, n, k, ja, sigma, u,
+                           p, x, warp, lane, &s_part[rg][warp]);
+        __syncthreads();
+        if (warp == 0) {
+            // ---- 3. publish the products and the next column, arrive, wait
+            double2* out = o.qa + (size_t)((k + 1) & 1) * n;
+            for (int r = lane; r < R; r += 32) {
+                const int i = g + (rf + r) * G;
+                const double* q = s_part[r];
+                const double* row = r >= rg ? rows + (size_t)(rf + r - rs0) * ldn : o.F + (size_t)i * n;
+                __stcg(out + i, make_double2(((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7])),
+                                             row[k + 1]));
+            }
+            __syncwarp();
+            target += (unsigned)min(G, n - 1 - k);
+            if (lane == 0) {
+                int ok = 1;
+                if (G > 1) {
+                    sk_atom_add_release(o.ctr, 1u);
+                    unsigned polls = 0;
+                    while (sk_ld_acquire(o.ctr) < target) {
+                        ++polls;
+                        if (polls > o.cap || ((polls & 255u) == 0 && *(volatile int*)o.status != 0)) {
+                            ok = 0;
+                            break;
+                        }
+                        if (polls > 256) __nanosleep(64);
+                    }
+                    if (!ok) sk_set_error(o.status, SKEW_ERR_DEVICE_TIMEOUT);
+                }
+                s_ok = ok;
+            }
+        } else if (warp >= 4) {
+            // ---- meanwhile: the norm of x below its first element, beta and
+            // sigma (H = I - sigma u u^T, sigma = 2 / |u|^2 = -1 / (beta u_0))
+            double nr = 0.0;
+            for (int j = k + 2 + (t - 128); j < n; j += 128) nr = fma(x[j], x[j], nr);
+            nr = sk_warp_sum(nr);
+            if (lane == 0) s_red[warp - 4] = nr;
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (warp == 4 && lane == 0) {
+                const double s2 = (s_red[0] + s_red[1]) + (s_red[2] + s_red[3]);
+                const double x0 = x[k + 1];
+                double b = x0, sg = 0.0, inv = 0.0;
+                if (s2 != 0.0) {
+                    const double rr = sqrt(fma(x0, x0, s2));
+                    b = (x0 >= 0.0) ? -rr : rr;
+                    sg = -1.0 / (b * (x0 - b));
+                    inv = -sg * b;
+                }
+                s_sc[0] = b;
+                s_sc[1] = sg;
+                s_sc[2] = inv;
+                s_sc[3] = x0 - b;
+            }
+        }
+        __syncthreads();
+        if (!s_ok) return;
+        beta = s_sc[0];
+        sigma = s_sc[1];
+        // ---- the reflector out, scaled to a unit leading element
+        {
+            const double inv = s_sc[2], u0 = s_sc[3];
+            for (int r = t; r < R; r += OT) {
+                const int i = g + (rf + r) * G;
+                o.V[(size_t)k * n + i] = (i == k + 1) ? 1.0 : x[i] * inv;
+            }
+            if (ilast == n - 1 && t == 0) {
+                o.tau[k] = sigma * u0 * u0;
+                o.alpha[k] = -beta;
+            }
+            if (t == 0) x[k + 1] = u0;  // x_0 itself is not read above
+            double* sw = u;
+            u = x;
+            x = sw;
+        }
+        __syncthreads();
+    }
+}
+
+// Full skew matrix by rows from the strict lower triangle of A (column-major):
+// F[i * n + j] = A(i, j) below the diagonal, -A(j, i) above.  32 x 32 tiles
+// through shared memory, both sides coalesced.
+__global__ void __launch_bounds__(256)
+os_full_kernel(int n, const double* __restrict__ A, int lda, double* __restrict__ F, int check, int* status) {
+    __shared__ double tile[32][33];
+    const int bi = blockIdx.x * 32, bj = blockIdx.y * 32;
+    if (bi < bj) return;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    bool bad = false;
+    for (int jj = ty; jj < 32; jj += 8) {
+        const int i = bi + tx, j = bj + jj;
+        double v = 0.0;
+        if (i < n && j < n && i > j) {
+            v = A[(size_t)j * lda + i];
+            if (check && !isfinite(v)) bad = true;
+        }
+        tile[jj][tx] = v;
+        // F(j, i) = -A(i, j); the diagonal and the part above it of a diagonal tile come below
+        if (i < n && j < n && i > j) F[(size_t)j * n + i] = -v;
+        if (i < n && i == j) F[(size_t)j * n + i] = 0.0;
+    }
+    __syncthreads();
+    for (int ii = ty; ii < 32; ii += 8) {
+        const int i = bi + ii, j = bj + tx;
+        if (i < n && j < n && i > j) F[(size_t)i * n + j] = tile[tx][ii];
+    }
+    if (bad) sk_set_error(status, SKEW_ERR_NONFINITE);
+}
+
+// ---- back-transformation: Z <- H_0 H_1 ... H_{n-3} Z ------------------------
+// Panels of 64 reflectors (the last one padded with zero columns) act as one
+// compact WY block (Eq. 7).  T is not formed: T^-1 = diag(1 / tau) + the strict
+// upper triangle of V^T V, so T y is a back substitution with V^T V.
+
+constexpr int GR = 256;  // rows of one Gram partial
+constexpr int PB = 64;   // reflectors per panel
+
+// Upper triangle of V_p^T V_p over GR rows: CTA (p, s), 136 threads with one
+// 4 x 4 tile each.  part: [s][p][column][row].
+__global__ void __launch_bounds__(160)
+os_gram_kernel(int n, const double* __restrict__ V, int ldv, double* __restrict__ part) {
+    const int p = blockIdx.x, s = blockIdx.y, P = gridDim.x, t = threadIdx.x;
+    const int o = p * PB + 1, lo = o + s * GR, hi = min(n, lo + GR);
+    if (lo >= n) return;
+    __shared__ double vs[PB][33];
+    int ti = 0, tj = 0;
+    if (t < 136) {
+        int e = t;  // tile (ti, tj), ti <= tj
+        while (e > tj) e -= ++tj;
+        ti = e;
+    }
+    double acc[4][4] = {};
+    for (int r0 = lo; r0 < hi; r0 += 32) {
+        for (int e = t; e < PB * 32; e += 160) {
+            const int r = e & 31, c = e >> 5;
+            vs[c][r] = (r0 + r < hi) ? V[(size_t)(p * PB + c) * ldv + r0 + r] : 0.0;
+        }
+        __syncthreads();
+        if (t < 136) {
+#pragma unroll 4
+            for (int r = 0; r < 32; r++) {
+                double a[4], b[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) a[i] = vs[4 * ti + i][r], b[i] = vs[4 * tj + i][r];
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+#pragma unroll
+                    for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            }
+        }
+        __syncthreads();
+    }
+    if (t < 136) {
+        double* q = part + ((size_t)s * P + p) * PB * PB;
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) q[(size_t)(4 * tj + j) * PB + 4 * ti + i] = acc[i][j];
+    }
+}
+
+// Sums the partials in order.  scaled: Gt[p][i][l] = (V^T V)_{l i} tau_i for
+// l < i, 0 elsewhere (the back substitution's rows); else the plain upper
+// triangle, mirrored.
+__global__ void __launch_bounds__(256)
+os_gram_sum_kernel(int n, const double* __restrict__ part, const double* __restrict__ tau, double* __restrict__ Gt,
+                   int scaled) {
+    const int p = blockIdx.x, P = gridDim.x;
+    const int m = n - (p * PB + 1), S = (m + GR - 1) / GR;
+    for (int e = blockIdx.y * 256 + threadIdx.x; e < PB * PB; e += gridDim.y * 256) {
+        const int l = e % PB, i = e / PB;
+        double g = 0.0;
+        if (l < i || (!scaled && l == i))
+            for (int s = 0; s < S; s++) g += part[((size_t)s * P + p) * PB * PB + e];
+        if (scaled) {
+            Gt[(size_t)p * PB * PB + e] = g * tau[p * PB + i];
+        } else if (l <= i) {
+            Gt[(size_t)p * PB * PB + e] = g;
+            Gt[(size_t)p * PB * PB + (size_t)l * PB + i] = g;
+        }
+    }
+}
+
+constexpr int WT = 256;  // threads of the WY kernel
+
+// One CTA carries E eigenvectors (C = 2 E columns: real and imaginary parts)
+// through every panel without leaving the SM: the slab of Z stays in shared
+// memory, V streams from L2 (read twice per panel), and nothing is exchanged
+// between CTAs.  The D map is applied on the way in (Algorithm 1 step 3) and the parts
+// go straight to Z_re / Z_im.  Bound by the FP64 pipe: 2 FMA per element of
+// V and column.
+template <int E>
+__global__ void __launch_bounds__(WT, 1)
+os_wy_kernel(int n, int nev, const double* __restrict__ V, const double* __restrict__ Gt,
+             const double* __restrict__ tau, const double* __restrict__ Qi, double* __restrict__ Zre,
+             double* __restrict__ Zim, int ldz) {
+    constexpr int C = 2 * E, VG = C <= 8 ? 8 : 4, NP = 8 / VG;
+    constexpr int NW = WT / 32;
+    extern __shared__ __align__(16) double wy_sm[];
+    double* ys = wy_sm;              // [64][C]
+    double* gs = ys + PB * C;        // [64][64]
+    double* zs = gs + PB * PB;       // [C][n]
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int e0 = blockIdx.x * E;
+    // D q: rows r mod 4 = 0, 1, 2, 3 of q are times 1, i, -1, -i
+    for (int i = t; i < n; i += WT) {
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+            double q = e0 + e < nev ? Qi[(size_t)i * nev + e0 + e] : 0.0;
+            if (i & 2) q = -q;
+            zs[(size_t)(2 * e) * n + i] = (i & 1) ? 0.0 : q;
+            zs[(size_t)(2 * e + 1) * n + i] = (i & 1) ? q : 0.0;
+        }
+    }
+    const int P = (n - 2 + PB - 1) / PB;
+    for (int p = P - 1; p >= 0; p--) {
+        const int o = p * PB + 1;
+        const double* Vp = V + (size_t)p * PB * n;
+        for (int e = t; e < PB * PB; e += WT) gs[e] = Gt[(size_t)p * PB * PB + e];
+        __syncthreads();
+        // Y = V_p^T Z: a warp takes 8 columns of V, lanes the rows
+#pragma unroll 1
+        for (int pass = 0; pass < NP; pass++) {
+            const int v0 = warp * 8 + pass * VG;
+            const double* Vc = Vp + (size_t)v0 * n;
+            double acc[VG * C];
+#pragma unroll
+            for (int i = 0; i < VG * C; i++) acc[i] = 0.0;
+            double vv[VG], vn[VG];
+            int r = o + lane;
+#pragma unroll
+            for (int i = 0; i < VG; i++) vn[i] = r < n ? Vc[(size_t)i * n + r] : 0.0;
+            for (; r - lane < n; r += 32) {
+#pragma unroll
+                for (int i = 0; i < VG; i++) {
+                    vv[i] = vn[i];
+                    vn[i] = r + 32 < n ? Vc[(size_t)i * n + r + 32] : 0.0;
+                }
+                const int rr = r < n ? r : n - 1;
+#pragma unroll
+                for (int c = 0; c < C; c++) {
+                    const double z = zs[(size_t)c * n + rr];
+#pragma unroll
+                    for (int i = 0; i < VG; i++) acc[i * C + c] = fma(vv[i], z, acc[i * C + c]);
+                }
+            }
+            WarpSums<VG * C> ws;
+            ws.run(acc, lane);
+#pragma unroll
+            for (int i = 0; i < WarpSums<VG * C>::H5; i++)
+                if (i < ws.cnt) ys[v0 * C + ws.first + i] = acc[i];
+        }
+        __syncthreads();
+        // y <- T y by back substitution, one warp per column
+        for (int c = warp; c < C; c += NW) {
+            double y0 = ys[lane * C + c], y1 = ys[(lane + 32) * C + c];
+#pragma unroll 4
+            for (int i = 63; i >= 32; i--) {
+                const double b = __shfl_sync(0xffffffffu, y1, i - 32);
+                y1 = fma(-gs[i * PB + lane + 32], b, y1);
+                y0 = fma(-gs[i * PB + lane], b, y0);
+            }
+#pragma unroll 4
+            for (int i = 31; i > 0; i--) {
+                const double b = __shfl_sync(0xffffffffu, y0, i);
+                y0 = fma(-gs[i * PB + lane], b, y0);
+            }
+            ys[lane * C + c] = -tau[p * PB + lane] * y0;
+            ys[(lane + 32) * C + c] = -tau[p * PB + lane + 32] * y1;
+        }
+        __syncthreads();
+        // Z -= V_p y: warps take blocks of 32 rows
+        for (int rb = warp; o + 32 * rb < n; rb += NW) {
+            const int r = o + 32 * rb + lane, rr = r < n ? r : n - 1;
+            double z[C];
+#pragma unroll
+            for (int c = 0; c < C; c++) z[c] = zs[(size_t)c * n + rr];
+            const double* Vr = Vp + rr;
+            double vn[8];
+#pragma unroll
+            for (int i = 0; i < 8; i++) vn[i] = Vr[(size_t)i * n];
+            for (int v = 0; v < PB; v += 8) {
+                double vv[8];
+                const int nx = v + 8 < PB ? v + 8 : v;
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+                    vv[i] = vn[i];
+                    vn[i] = Vr[(size_t)(nx + i) * n];
+                }
+#pragma unroll
+                for (int i = 0; i < 8; i++)
+#pragma unroll
+                    for (int c = 0; c < C; c += 2) {
+                        const double2 y = *reinterpret_cast<const double2*>(ys + (v + i) * C + c);
+                        z[c] = fma(vv[i], y.x, z[c]);
+                        z[c + 1] = fma(vv[i], y.y, z[c + 1]);
+                    }
+            }
+            if (r < n) {
+#pragma unroll
+                for (int c = 0; c < C; c++) zs[(size_t)c * n + r] = z[c];
+            }
+        }
+        __syncthreads();
+    }
+    for (int e = 0; e < E && e0 + e < nev; e++)
+        for (int i = t; i < n; i += WT) {
+            Zre[(size_t)(e0 + e) * ldz + i] = zs[(size_t)(2 * e) * n + i];
+            Zim[(size_t)(e0 + e) * ldz + i] = zs[(size_t)(2 * e + 1) * n + i];
+        }
+}
+
+size_t wy_smem(int n, int E) { return sizeof(double) * ((size_t)PB * 2 * E + PB * PB + 2 * (size_t)E * n); }
+
+template <int E>
+cudaError_t wy_launch(cudaStream_t st, int n, int nev, const double* V, const double* Gt, const double* tau,
+                      const double* Qi, double* Zre, double* Zim, int ldz) {
+    const size_t dyn = wy_smem(n, E);
+    if (const cudaError_t e = cudaFuncSetAttribute(os_wy_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn))
+        return e;
+    os_wy_kernel<E><<<(nev + E - 1) / E, WT, dyn, st>>>(n, nev, V, Gt, tau, Qi, Zre, Zim, ldz);
+    count_launch();
+    return cudaGetLastError();
+}
+
+int os_srows(int n, int G) {
+    const int rmax = (n + G - 1) / G;
+    const size_t vec = 3 * sizeof(double) * (size_t)(n | 1), row = sizeof(double) * (size_t)(n | 1);
+    const size_t cap = 222 * 1024;  // of 227 KB: the static arrays take about 4.3 KB
+    const int fit = vec + row > cap ? 0 : (int)((cap - vec) / row);
+    return std::min(rmax, fit);
+}
+
+}  // namespace
+
+int onestep_max() { return std::min(OMAXR * device_sms(), 9000); }
+
+size_t onestep_ws(int n) {
+    Carve cv(nullptr, ~size_t(0));
+    cv.take<double2>(2 * (size_t)(n > 0 ? n : 1));
+    cv.take<unsigned>(16);
+    return cv.off + 256;
+}
+
+int onestep_vcols(int n) { return n > 2 ? (n - 2 + 63) / 64 * 64 : 64; }
+
+cudaError_t onestep_full(cudaStream_t st, int n, const double* A, int lda, double* F, int check, int* status) {
+    const int nb = (n + 31) / 32;
+    os_full_kernel<<<dim3(nb, nb), 256, 0, st>>>(n, A, lda, F, check, status);
+    count_launch();
+    return cudaGetLastError();
+}
+
+int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, double* alpha, void* ws,
+                   size_t ws_bytes, int* d_status, unsigned spin_cap) {
+    if (n < 2) return 0;
+    Carve cv(ws, ws_bytes);
+    OsArgs o{};
+    o.qa = cv.take<double2>(2 * (size_t)n);
+    o.ctr = cv.take<unsigned>(16);
+    if (!cv.ok) return SKEW_ERR_WORKSPACE;
+    const size_t vc = (size_t)onestep_vcols(n);
+    if (const cudaError_t e = cudaMemsetAsync(V, 0, sizeof(double) * vc * n, st)) return cuda_fail(e);
+    if (const cudaError_t e = cudaMemsetAsync(tau, 0, sizeof(double) * vc, st)) return cuda_fail(e);
+    if (const cudaError_t e = cudaMemsetAsync(o.ctr, 0, sizeof(unsigned), st)) return cuda_fail(e);
+    // two rows per CTA and more
+    const int G = std::min(device_sms(), (n + 1) / 2);
+    if (n > OMAXR * G) return SKEW_ERR_UNSUPPORTED;
+    o.n = n;
+    o.F = F;
+    o.V = V;
+    o.tau = tau;
+    o.alpha = alpha;
+    o.status = d_status;
+    o.cap = spin_cap ? spin_cap : SK_SPIN_CAP;
+    o.srows = os_srows(n, G);
+    const size_t dyn = sizeof(double) * (size_t)(n | 1) * (3 + (size_t)o.srows);
+    if (const cudaError_t e =
+            cudaFuncSetAttribute(onestep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn))
+        return cuda_fail(e);
+    void* args[] = {&o};
+    KtScope kt(st, KT_PANEL_QR);
+    const cudaError_t e = cudaLaunchCooperativeKernel((void*)onestep_kernel, dim3(G), dim3(OT), args, dyn, st);
+    count_launch();
+    if (e == cudaErrorCooperativeLaunchTooLarge) return SKEW_ERR_LAUNCH;
+    return cuda_ok(e);
+}
+
+// Eigenvectors of one wave in shared memory: every CTA one slab.
+static int wy_e(int n, int nev) {
+    const int sms = device_sms();
+    const int e = (nev + sms - 1) / sms;
+    return (e <= 6 && wy_smem(n, e) <= 226 * 1024) ? e : 0;
+}
+
+bool onestep_wy_fits(int n, int nev) { return wy_e(n, nev) > 0; }
+
+size_t onestep_back_ws(int n) {
+    const size_t P = (size_t)(onestep_vcols(n) / PB), S = (size_t)((n + GR - 1) / GR);
+    Carve cv(nullptr, ~size_t(0));
+    cv.take<double>(P * S * PB * PB);
+    cv.take<double>(P * PB * PB);
+    return cv.off + 256;
+}
+
+namespace {
+// V^T V of every panel (os_gram_sum_kernel's two forms)
+cudaError_t os_gram(cudaStream_t st, int n, const double* V, const double* tau, double* part, double* G, int scaled) {
+    const int P = (n - 2 + PB - 1) / PB, S = (n - 1 + GR - 1) / GR;
+    os_gram_kernel<<<dim3(P, S), 160, 0, st>>>(n, V, n, part);
+    os_gram_sum_kernel<<<dim3(P, 4), 256, 0, st>>>(n, part, tau, G, scaled);
+    count_launch(2);
+    return cudaGetLastError();
+}
+}  // namespace
+
+int onestep_back(cudaStream_t st, int n, int nev, const double* V, const double* tau, const double* Qi, double* Zre,
+                 double* Zim, int ldz, void* ws, size_t ws_bytes) {
+    const int E = wy_e(n, nev);
+    if (E <= 0) return SKEW_ERR_UNSUPPORTED;
+    const size_t P = (size_t)(onestep_vcols(n) / PB), S = (size_t)((n + GR - 1) / GR);
+    Carve cv(ws, ws_bytes);
+    double* part = cv.take<double>(P * S * PB * PB);
+    double* Gt = cv.take<double>(P * PB * PB);
+    if (!cv.ok) return SKEW_ERR_WORKSPACE;
+    KtScope kt(st, KT_GEMM_F64);
+    if (n > 2) {
+        if (const cudaError_t e = os_gram(st, n, V, tau, part, Gt, 1)) return cuda_fail(e);
+    }
+    cudaError_t e;
+    switch (E) {
+    case 1: e = wy_launch<1>(st, n, nev, V, Gt, tau, Qi, Zre, Zim, ldz); break;
+    case 2: e = wy_launch<2>(st, n, nev, V, Gt, tau, Qi, Zre, Zim, ldz); break;
+    case 3: e = wy_launch<3>(st, n, nev, V, Gt, tau, Qi, Zre, Zim, ldz); break;
+    case 4: e = wy_launch<4>(st, n, nev, V, Gt, tau, Qi, Zre, Zim, ldz); break;
+    case 5: e = wy_launch<5>(st, n, nev, V, Gt, tau, Qi, Zre, Zim, ldz); break;
+    default: e = wy_launch<6>(st, n, nev, V, Gt, tau, Qi, Zre, Zim, ldz); break;
+    }
+    return cuda_ok(e);
+}
+
+int onestep_tfactors(cudaStream_t st, int n, const double* V, const double* tau, double* Tfac, void* ws,
+                     size_t ws_bytes) {
+    if (n < 3) return 0;
+    const size_t P = (size_t)(onestep_vcols(n) / PB), S = (size_t)((n + GR - 1) / GR);
+    Carve cv(ws, ws_bytes);
+    double* part = cv.take<double>(P * S * PB * PB);
+    double* G = cv.take<double>(P * PB * PB);
+    if (!cv.ok) return SKEW_ERR_WORKSPACE;
+    KtScope kt(st, KT_GEMM_F64);
+    if (const cudaError_t e = os_gram(st, n, V, tau, part, G, 0)) return cuda_fail(e);
+    return cuda_ok(tfactor_panels(st, (int)P, tau, G, Tfac));
+}
+
+}  // namespace sk

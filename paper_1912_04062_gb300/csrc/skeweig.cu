@@ -43,6 +43,25 @@ __global__ void split_z_kernel(int n, int nev, const double* __restrict__ Z, int
     }
 }
 
+// Columns k and nev + k of Z (real and imaginary part of vector k) scaled to
+// a unit vector in FP64.  The double-float inverse iteration leaves norms off
+// by FP32 rounding; the refinement's first-order correction would keep the
+// square of that.
+__global__ void __launch_bounds__(256) unit_columns_kernel(int n, int nev, double* __restrict__ Z) {
+    __shared__ double red[32];
+    double* x = Z + (size_t)blockIdx.x * n;
+    double* y = x + (size_t)nev * n;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) s = fma(x[i], x[i], fma(y[i], y[i], s));
+    s = sk_block_sum(s, red);
+    if (!(s > 0.0)) return;
+    const double f = 1.0 / sqrt(s);
+    for (int i = threadIdx.x; i < n; i += 256) {
+        x[i] *= f;
+        y[i] *= f;
+    }
+}
+
 __global__ void store_status_kernel(const int* status, int* d_info) {
     if (threadIdx.x == 0) *d_info = *status;
 }
@@ -79,7 +98,16 @@ struct Plan {
     void *ws_reduce, *ws_chase, *ws_tri, *ws_qband, *ws_refine, *ws_qtc;
     size_t sz_reduce, sz_chase, sz_tri, sz_qband, sz_refine, sz_qtc;
     bool refine;  // mixed form with a complete basis (n even, nev = n/2)
+    bool onestep;  // direct tridiagonalisation instead of band + chase (onestep.cu)
+    bool wy;       // its FP64 back-transformation in one launch (else panel products)
+    double *V1, *tau1;  // its reflectors
+    void *ws_one, *ws_back;
+    size_t sz_one, sz_back;
 };
+
+// Orders that take the direct reduction (measured limits: see make_plan).
+constexpr int ONESTEP_FP64 = 8192, ONESTEP_FP64_VALUES = 5500, ONESTEP_REFINE = 4200, ONESTEP_PARTIAL = 5000,
+              ONESTEP_VALUES = 3800;
 
 // One carve-up routine serves both sizing (base == nullptr) and placement.
 bool carve_plan(Plan& p, Carve& cv) {
@@ -87,6 +115,31 @@ bool carve_plan(Plan& p, Carve& cv) {
     const size_t nn = n ? n : 1;
     p.status = cv.take<int>(16);
     p.W = cv.take<double>(nn * nn);
+    if (p.onestep) {
+        const size_t vc = (size_t)onestep_vcols(p.n), ne = (size_t)(p.nev ? p.nev : 1);
+        p.V1 = cv.take<double>(vc * nn);
+        p.tau1 = cv.take<double>(vc);
+        p.alpha = cv.take<double>(nn);
+        p.Qi = p.vectors ? cv.take<double>(nn * ne) : nullptr;
+        p.sz_one = onestep_ws(p.n);
+        p.ws_one = cv.take<char>(p.sz_one);
+        p.sz_tri = tridiag_ws(p.n, p.nev);
+        p.ws_tri = cv.take<char>(p.sz_tri);
+        if (p.vectors) {
+            p.sz_back = onestep_back_ws(p.n);
+            p.ws_back = cv.take<char>(p.sz_back);
+            if (!p.wy) {
+                p.Z = cv.take<double>(nn * 2 * ne);
+                p.Tfac = cv.take<double>(vc * b);
+                p.sz_qband = p.mixed ? qband_mixed_ws(p.n, p.b, 2 * p.nev, p.qband_prec)
+                                     : qband_ws(p.n, p.b, 2 * p.nev);
+                p.ws_qband = cv.take<char>(p.sz_qband);
+            }
+        }
+        p.sz_refine = p.refine ? refine_ws(p.n) : 0;
+        p.ws_refine = p.refine ? cv.take<char>(p.sz_refine) : nullptr;
+        return cv.ok;
+    }
     p.Tfac = cv.take<double>((size_t)(p.P ? p.P : 1) * b * b);
     p.ldab = 2 * b + 1;
     p.AB = cv.take<double>(p.ldab * nn);
@@ -163,6 +216,14 @@ Plan make_plan(int n, int nev, const skew_opts* o, bool vectors) {
     // with 8.  Without refinement they stay FP64-accurate.
     p.reduce_slices = p.refine ? 6 : 8;
     p.qband_slices = p.refine ? 5 : 8;
+    const int lim = !p.mixed ? (vectors ? ONESTEP_FP64 : ONESTEP_FP64_VALUES)
+                             : (p.refine ? ONESTEP_REFINE : vectors ? ONESTEP_PARTIAL : ONESTEP_VALUES);
+    // a request for a Q_trd arithmetic keeps the two-step route that has one,
+    // unless it names the mode's own choice
+    const bool any_qtrd = !o || o->qtrd == SKEW_QTRD_AUTO ||
+                          (refined_mode && vectors && !p.refine && o->qtrd == SKEW_QTRD_DF);
+    p.onestep = p.b == 64 && (!p.mixed || refined_mode) && any_qtrd && n >= 2 && n <= lim && n <= onestep_max();
+    p.wy = p.onestep && vectors && !p.mixed && onestep_wy_fits(n, nev);
     return p;
 }
 
@@ -216,89 +277,132 @@ int run_solve(cudaStream_t st, int n, const double* A, int lda, int nev, double*
     last_refine_info() = RefineInfo{};  // iterations = 0 unless this solve refines
 
     mark(0);
-    {
-        KtScope kt(st, KT_OTHER);
-        zero_int_kernel<<<1, 32, 0, st>>>(p.status);
-        copy_lower_kernel<<<grid_for((size_t)n * n), 256, 0, st>>>(n, A, lda, p.W, n, o ? o->check_finite : 0,
-                                                                   p.status);
-    }
-    count_launch(2);
-    mark(1);
-    int rc = band_reduce(st, n, p.W, n, p.b, p.Tfac, p.ws_reduce, p.sz_reduce, p.status, p.reduce_prec,
-                         p.reduce_slices, spin_cap);
-    if (rc) return rc;
-    mark(2);
-    if (band_pack(st, n, p.b, p.W, n, p.AB, (int)p.ldab) != cudaSuccess) return SKEW_ERR_CUDA;
-    mark(3);
-    if (p.tau32) {
-        // FP32 reflector copies for Q_trd: the taus of steps a sweep does not
-        // have stay zero (the FP64 copies are not needed then)
-        const size_t nsw64 = ((size_t)p.nsw + 63) / 64 * 64;
-        if (const cudaError_t e = cudaMemsetAsync(p.tau32, 0, sizeof(float) * (size_t)p.K * nsw64, st))
-            return cuda_fail(e);
-        rc = chase(st, n, p.b, p.AB, (int)p.ldab, p.alpha, nullptr, nullptr, p.ws_chase, p.sz_chase, p.status,
-                   spin_cap, p.V32, p.tau32);
-    } else {
-        rc = chase(st, n, p.b, p.AB, (int)p.ldab, p.alpha, p.Vtrd, p.tautrd, p.ws_chase, p.sz_chase, p.status,
-                   spin_cap);
-    }
-    if (rc) return rc;
-    mark(4);
-    // with refinement the eigenvalues are recomputed from the Rayleigh
-    // quotients: the double-float brackets suffice to start from
-    rc = tridiag_eig(st, n, p.alpha, nev, lambda, vectors ? p.Qi : nullptr, p.ws_tri, p.sz_tri, p.status, maxit,
-                     !p.refine, !(o && o->tridiag == SKEW_TRIDIAG_FULL));
-    if (rc) return rc;
-    mark(5);
-    if (vectors) {
-        // Algorithm 1 step 3 (D map) fused with the interleaved -> column-major
-        // move; Z = [X | Y] is n x 2 nev with leading dimension n.
-        KtScope kt(st, KT_OTHER);
-        if (interleaved_to_colmajor(st, n, nev, p.Qi, p.Z, p.Z + (size_t)n * nev, n, true) != cudaSuccess)
-            return SKEW_ERR_CUDA;
-    }
-    mark(6);
-    if (vectors && p.qtrd_df) {
-        if (apply_qtrd_df(st, n, p.b, p.Vtrd, p.tautrd, p.Z, n, 2 * nev, p.status) != cudaSuccess)
-            return SKEW_ERR_CUDA;
-    } else if (vectors && !p.qtrd_f32) {
-        if (apply_qtrd(st, n, p.b, p.Vtrd, p.tautrd, p.Z, n, 2 * nev) != cudaSuccess) return SKEW_ERR_CUDA;
-    } else if (vectors) {
-        // mixed form: Q_trd in FP32 arithmetic (the chase's FP32 reflector copies)
-        const size_t cnt = (size_t)n * 2 * nev;
+    if (p.onestep) {
+        const int check = o ? o->check_finite : 0;
         {
             KtScope kt(st, KT_OTHER);
-            f64_to_f32_kernel<<<grid_for(cnt), 256, 0, st>>>(cnt, p.Z, p.Z32);
+            zero_int_kernel<<<1, 32, 0, st>>>(p.status);
+            count_launch();
+            if (const cudaError_t e = onestep_full(st, n, A, lda, p.W, check, p.status)) return cuda_fail(e);
         }
-        count_launch();
-        if (p.qtrd_tc) {
-            rc = apply_qtrd_tc(st, n, p.V32, p.tau32, p.Z32, n, 2 * nev, p.ws_qtc, p.sz_qtc, p.status);
-            if (rc) return rc;
-        } else if (apply_qtrd_f32(st, n, p.b, p.V32, p.tau32, p.Z32, n, 2 * nev, p.status) != cudaSuccess) {
-            return SKEW_ERR_CUDA;
-        }
-        {
-            KtScope kt(st, KT_OTHER);
-            f32_to_f64_kernel<<<grid_for(cnt), 256, 0, st>>>(cnt, p.Z32, p.Z);
-        }
-        count_launch();
-    }
-    mark(7);
-    if (vectors) {
-        rc = p.mixed ? apply_qband_mixed(st, n, p.b, p.W, n, p.Tfac, p.Z, n, 2 * nev, p.ws_qband, p.sz_qband, p.status,
-                                         p.qband_prec, p.qband_slices)
-                     : apply_qband(st, n, p.b, p.W, n, p.Tfac, p.Z, n, 2 * nev, p.ws_qband, p.sz_qband);
+        mark(1);
+        int rc = onestep_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap);
         if (rc) return rc;
+        mark(2);
+        mark(3);
+        mark(4);
+        rc = tridiag_eig(st, n, p.alpha, nev, lambda, vectors ? p.Qi : nullptr, p.ws_tri, p.sz_tri, p.status, maxit,
+                         !p.refine, !(o && o->tridiag == SKEW_TRIDIAG_FULL));
+        if (rc) return rc;
+        mark(5);
+        if (vectors && !p.wy) {
+            KtScope kt(st, KT_OTHER);
+            if (interleaved_to_colmajor(st, n, nev, p.Qi, p.Z, p.Z + (size_t)n * nev, n, true) != cudaSuccess)
+                return SKEW_ERR_CUDA;
+            if (p.refine) {
+                unit_columns_kernel<<<nev, 256, 0, st>>>(n, nev, p.Z);
+                count_launch();
+            }
+        }
+        mark(6);
+        mark(7);
+        if (vectors && p.wy) {
+            rc = onestep_back(st, n, nev, p.V1, p.tau1, p.Qi, Zre, Zim, ldz, p.ws_back, p.sz_back);
+            if (rc) return rc;
+        } else if (vectors && n > 2) {
+            rc = onestep_tfactors(st, n, p.V1, p.tau1, p.Tfac, p.ws_back, p.sz_back);
+            if (!rc)
+                rc = p.mixed ? apply_qband_mixed(st, n, p.b, p.V1, n, p.Tfac, p.Z, n, 2 * nev, p.ws_qband, p.sz_qband,
+                                                 p.status, p.qband_prec, p.qband_slices, true)
+                             : apply_qband(st, n, p.b, p.V1, n, p.Tfac, p.Z, n, 2 * nev, p.ws_qband, p.sz_qband, true);
+            if (rc) return rc;
+        }
+    } else {
+        {
+            KtScope kt(st, KT_OTHER);
+            zero_int_kernel<<<1, 32, 0, st>>>(p.status);
+            copy_lower_kernel<<<grid_for((size_t)n * n), 256, 0, st>>>(n, A, lda, p.W, n, o ? o->check_finite : 0,
+                                                                       p.status);
+        }
+        count_launch(2);
+        mark(1);
+        int rc = band_reduce(st, n, p.W, n, p.b, p.Tfac, p.ws_reduce, p.sz_reduce, p.status, p.reduce_prec,
+                             p.reduce_slices, spin_cap);
+        if (rc) return rc;
+        mark(2);
+        if (band_pack(st, n, p.b, p.W, n, p.AB, (int)p.ldab) != cudaSuccess) return SKEW_ERR_CUDA;
+        mark(3);
+        if (p.tau32) {
+            // FP32 reflector copies for Q_trd: the taus of steps a sweep does not
+            // have stay zero (the FP64 copies are not needed then)
+            const size_t nsw64 = ((size_t)p.nsw + 63) / 64 * 64;
+            if (const cudaError_t e = cudaMemsetAsync(p.tau32, 0, sizeof(float) * (size_t)p.K * nsw64, st))
+                return cuda_fail(e);
+            rc = chase(st, n, p.b, p.AB, (int)p.ldab, p.alpha, nullptr, nullptr, p.ws_chase, p.sz_chase, p.status,
+                       spin_cap, p.V32, p.tau32);
+        } else {
+            rc = chase(st, n, p.b, p.AB, (int)p.ldab, p.alpha, p.Vtrd, p.tautrd, p.ws_chase, p.sz_chase, p.status,
+                       spin_cap);
+        }
+        if (rc) return rc;
+        mark(4);
+        // with refinement the eigenvalues are recomputed from the Rayleigh
+        // quotients: the double-float brackets suffice to start from
+        rc = tridiag_eig(st, n, p.alpha, nev, lambda, vectors ? p.Qi : nullptr, p.ws_tri, p.sz_tri, p.status, maxit,
+                         !p.refine, !(o && o->tridiag == SKEW_TRIDIAG_FULL));
+        if (rc) return rc;
+        mark(5);
+        if (vectors) {
+            // Algorithm 1 step 3 (D map) fused with the interleaved -> column-major
+            // move; Z = [X | Y] is n x 2 nev with leading dimension n.
+            KtScope kt(st, KT_OTHER);
+            if (interleaved_to_colmajor(st, n, nev, p.Qi, p.Z, p.Z + (size_t)n * nev, n, true) != cudaSuccess)
+                return SKEW_ERR_CUDA;
+        }
+        mark(6);
+        if (vectors && p.qtrd_df) {
+            if (apply_qtrd_df(st, n, p.b, p.Vtrd, p.tautrd, p.Z, n, 2 * nev, p.status) != cudaSuccess)
+                return SKEW_ERR_CUDA;
+        } else if (vectors && !p.qtrd_f32) {
+            if (apply_qtrd(st, n, p.b, p.Vtrd, p.tautrd, p.Z, n, 2 * nev) != cudaSuccess) return SKEW_ERR_CUDA;
+        } else if (vectors) {
+            // mixed form: Q_trd in FP32 arithmetic (the chase's FP32 reflector copies)
+            const size_t cnt = (size_t)n * 2 * nev;
+            {
+                KtScope kt(st, KT_OTHER);
+                f64_to_f32_kernel<<<grid_for(cnt), 256, 0, st>>>(cnt, p.Z, p.Z32);
+            }
+            count_launch();
+            if (p.qtrd_tc) {
+                rc = apply_qtrd_tc(st, n, p.V32, p.tau32, p.Z32, n, 2 * nev, p.ws_qtc, p.sz_qtc, p.status);
+                if (rc) return rc;
+            } else if (apply_qtrd_f32(st, n, p.b, p.V32, p.tau32, p.Z32, n, 2 * nev, p.status) != cudaSuccess) {
+                return SKEW_ERR_CUDA;
+            }
+            {
+                KtScope kt(st, KT_OTHER);
+                f32_to_f64_kernel<<<grid_for(cnt), 256, 0, st>>>(cnt, p.Z32, p.Z);
+            }
+            count_launch();
+        }
+        mark(7);
+        if (vectors) {
+            rc = p.mixed ? apply_qband_mixed(st, n, p.b, p.W, n, p.Tfac, p.Z, n, 2 * nev, p.ws_qband, p.sz_qband, p.status,
+                                             p.qband_prec, p.qband_slices)
+                         : apply_qband(st, n, p.b, p.W, n, p.Tfac, p.Z, n, 2 * nev, p.ws_qband, p.sz_qband);
+            if (rc) return rc;
+        }
     }
     mark(8);
     if (p.refine) {
         const int iters = (o && o->refine_iters > 0) ? (o->refine_iters < 8 ? o->refine_iters : 8) : 8;
         const double rho = (o && o->refine_rho > 0) ? (double)o->refine_rho : 1024.0;
-        rc = refine(st, n, A, lda, lambda, p.Z, iters, p.ws_refine, p.sz_refine, p.status, &last_refine_info(), rho);
+        const int rc =
+            refine(st, n, A, lda, lambda, p.Z, iters, p.ws_refine, p.sz_refine, p.status, &last_refine_info(), rho);
         if (rc) return rc;
     }
     mark(9);
-    if (vectors) {
+    if (vectors && !p.wy) {
         KtScope kt(st, KT_OTHER);
         split_z_kernel<<<grid_for((size_t)n * nev), 256, 0, st>>>(n, nev, p.Z, n, Zre, Zim, ldz);
         count_launch();

@@ -1,0 +1,96 @@
+"""The direct (one-step) reduction with its back-transformation, and the twisted
+eigenvectors of the tridiagonal, at the sizes where their tiling changes.
+
+Orders around a panel of 64 reflectors, around one, two and three rows per CTA
+of a 152-SM GPU, and the first one whose rows do not all fit shared memory;
+slabs of one to six eigenvectors per CTA.  The two-step route (an explicit FP64
+Q_trd) is the other side of the comparison.  Bounds: those of the other solve
+tests (1e-12 of the largest eigenvalue; residual and orthogonality 50 n eps).
+"""
+import numpy as np
+import pytest
+
+import inputs
+
+pytestmark = pytest.mark.gpu
+EPS = np.finfo(np.float64).eps
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _dev():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _solve(dA, nev, opts, vectors=True):
+    import torch
+    import paper_1912_04062_gb300 as sk
+    n = dA.shape[0]
+    ws = torch.empty(sk.workspace_size(n, nev, opts, vectors=vectors), dtype=torch.uint8, device="cuda")
+    lam = torch.empty(nev, dtype=torch.float64, device="cuda")
+    Zr = sk.fortran_empty(n, nev) if vectors else None
+    Zi = sk.fortran_empty(n, nev) if vectors else None
+    info = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    assert sk.skew_eig_ex(dA, nev, lam, Zr, Zi, ws, info, opts) == 0
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    return lam, Zr, Zi
+
+
+@pytest.mark.parametrize("n,nev", [(2, 1), (3, 1), (49, 24), (65, 32), (66, 33), (67, 1), (130, 65), (152, 3),
+                                   (153, 76), (305, 152), (306, 153), (459, 20), (610, 305), (914, 457),
+                                   (1825, 912), (1826, 40)])
+def test_direct_route_matches_two_step(n, nev):
+    import torch
+    import paper_1912_04062_gb300 as sk
+    A = inputs.random_skew(n, seed=7000 + n)
+    dA = sk.fortran(torch.from_numpy(A).cuda())
+    lam2, _, _ = _solve(dA, nev, sk.Options(qtrd=sk.SKEW_QTRD_FP64))
+    scale = float(lam2[0])
+    lam1, Zr, Zi = _solve(dA, nev, sk.Options())
+    assert float((lam1 - lam2).abs().max()) <= 1e-12 * scale
+    r, o, f = sk.metrics(dA, lam1, Zr, Zi)
+    assert r <= 50 * n * EPS * f and o <= 50 * n * EPS
+    # values only, and a second run, give the same bits
+    lam0, _, _ = _solve(dA, nev, sk.Options(), vectors=False)
+    assert torch.equal(lam0, lam1)
+    lam3, Zr3, Zi3 = _solve(dA, nev, sk.Options())
+    assert torch.equal(lam3, lam1) and torch.equal(Zr3, Zr) and torch.equal(Zi3, Zi)
+
+
+@pytest.mark.parametrize("n", [64, 307, 1002])
+def test_direct_route_refined_is_orthogonal(n):
+    # one refinement iteration follows the direct reduction: it has to leave
+    # the orthogonality of a converged refinement, not the square of the
+    # starting vectors' norm error
+    import torch
+    import paper_1912_04062_gb300 as sk
+    A = inputs.random_skew(n, seed=7100 + n)
+    dA = sk.fortran(torch.from_numpy(A).cuda())
+    lam, Zr, Zi = _solve(dA, n // 2, sk.Options(mode=sk.SKEW_MODE_MIXED_REFINED))
+    r, o, f = sk.metrics(dA, lam, Zr, Zi)
+    assert r <= 50 * n * EPS * f and o <= 5 * n * EPS
+
+
+@pytest.mark.parametrize("glue", [1e-3, 1e-6, 1e-9, 1e-13])
+@pytest.mark.parametrize("n", [62, 511])
+def test_twisted_vectors_of_glued_blocks(n, glue):
+    # equal blocks coupled by `glue`: pairs of eigenvalues about glue apart, so
+    # loose clusters (one Gram-Schmidt pass) and tight ones (iterated)
+    import torch
+    import paper_1912_04062_gb300 as sk
+    rng = np.random.default_rng(n)
+    h = (n - 1) // 2
+    half = rng.uniform(0.5, 2.0, h)
+    a = np.concatenate([half, [glue], half[::-1]])[: n - 1]
+    a = np.concatenate([a, rng.uniform(0.5, 2.0, n - 1 - a.size)])
+    nev = n // 2
+    da = torch.from_numpy(a).cuda()
+    lam, Q, st = sk.tridiag_eig(da, nev)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    S = torch.diag(da, 1) + torch.diag(da, -1)
+    scale = float(lam[0])
+    assert float((S @ Q - Q * lam).norm(dim=0).max()) <= 50 * n * EPS * scale
+    assert float((Q.T @ Q - torch.eye(nev, device="cuda", dtype=Q.dtype)).norm()) <= 50 * n * EPS
