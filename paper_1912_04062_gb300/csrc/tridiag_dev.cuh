@@ -13,7 +13,35 @@ namespace tri {
 struct TriScalars {
     double g;       // ||S||_1
     double pivmin;  // DBL_MIN * max(1, max alpha^2)
+    double down, up;  // powers of two: g down in [1, 2) (1 when g == 0), up = 1 / down
 };
+
+// 1 / d for 2^-1000 < |d| < 2^1000, within about one unit of the last place:
+// the hardware's FP32 reciprocal of the significand (2^-23), its exponent set
+// with integer operations, and one third-order Newton step y (1 + e + e^2),
+// e = 1 - d y.  Three FP64 instructions; the FP64 pipe issues one per 64
+// clocks and scheduler here, and the correctly rounded division takes nine
+// (640 clocks with its addition, measured).
+__device__ __forceinline__ double rcp_fast(double d) {
+    const int hi = __double2hiint(d), lo = __double2loint(d);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;"
+        : "=f"(r)
+        : "f"(__int_as_float(0x3f800000 | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29))));
+    const int rb = __float_as_int(r);
+    const int ex = (rb >> 23) - 127 + 1023 - (((hi >> 20) & 0x7ff) - 1023);
+    const double y = __hiloint2double((hi & (int)0x80000000) | (ex << 20) | ((rb & 0x7fffff) >> 3), rb << 29);
+    double e = fma(-d, y, 1.0);
+    e = fma(e, e, e);
+    return fma(y, e, y);
+}
+
+// Power of two that brings g > 0 into [1, 2).
+__device__ __forceinline__ double pow2_down(double g) {
+    int e;
+    frexp(g, &e);  // g = f 2^e, f in [1/2, 1)
+    return (g > 0.0 && isfinite(g)) ? ldexp(1.0, 1 - e) : 1.0;
+}
 
 __device__ __forceinline__ int sturm(int n, const double* __restrict__ a2, double pivmin, double x) {
     int cnt = 0;
@@ -62,6 +90,26 @@ __device__ __forceinline__ int bd_count(int m, const double* __restrict__ a2e, c
         if (fabs(d) < pivmin) d = -pivmin;
         cnt += (d < 0.0);
         sv = b2e[i] * sv / d - t;
+    }
+    return cnt;
+}
+
+// bd_count on the matrix scaled to g in [1, 2) (entries a2e, b2e <= 4), with
+// the quick reciprocal: six FP64 instructions a step.  A quotient off by a
+// unit of the last place is, like any rounding of the recurrence, a relative
+// perturbation of a_i and b_i.  Pivots below 2^-900 are raised to it.
+__device__ __forceinline__ int bd_count_scaled(int m, const double* __restrict__ a2e, const double* __restrict__ b2e,
+                                               double t) {
+    constexpr double PIV = 1.1830521861667747e-271;  // 2^-900
+    int cnt = 0;
+    double sv = -t;
+#pragma unroll 4
+    for (int i = 0; i < m; i++) {
+        double d = a2e[i] + sv;
+        const int e = (__double2hiint(d) >> 20) & 0x7ff;
+        if (e <= 123) d = -PIV;  // |d| < 2^-899
+        cnt += __double2hiint(d) < 0;
+        sv = fma(b2e[i] * sv, rcp_fast(d), -t);
     }
     return cnt;
 }
@@ -301,6 +349,174 @@ __device__ __forceinline__ void invit_cluster(int n, int nev, const double* __re
         if (!conv) atomicMin(fail, k);
         invit_sign(n, Q, ld, k);
     }
+}
+
+// ---- one eigenvector by a twisted factorisation ------------------------------
+// (Fernando, "On computing an eigenvector of a tridiagonal matrix", 1997;
+// Parlett and Dhillon 1997.)  With the pivots d+ of S - lambda I from the top
+// (d+_i = -lambda - alpha_{i-1} l+_{i-1}, l+_i = alpha_i / d+_i) and d- from the
+// bottom (l-_i = alpha_i / d-_{i+1}), gamma_i = -lambda - alpha_{i-1} l+_{i-1} -
+// alpha_i l-_i; at r = argmin |gamma_i| the vector z_r = 1, z_i = -l+_i z_{i+1}
+// above, z_{i+1} = -l-_i z_i below has residual |gamma_r| / |z| (no pivoting, no
+// start vector), and lambda + gamma_r / |z|^2 is its Rayleigh quotient.  Two
+// lanes a vector: lane half 0 runs downwards, half 1 upwards, the same
+// instructions on mirrored rows; sixteen vectors a warp.  as: alpha scaled to
+// g in [1, 2).
+constexpr int TW_IB = 8;
+
+// Reciprocal pivots Y (of row i) and ratios L (of edge i, i + 1) at shift lam,
+// this lane's direction.
+__device__ __forceinline__ void twist_factor(int n, const double* __restrict__ as, double lam, int half, double* Y,
+                                             double* L, size_t ld, int k, bool live) {
+    constexpr double PIV = 4.909093465297727e-91;  // 2^-300
+    double d = -lam;
+    for (int s0 = 0; s0 < n; s0 += TW_IB) {
+        double al[TW_IB];
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const int s = s0 + u;
+            al[u] = (s < n - 1) ? as[half ? n - 2 - s : s] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const int s = s0 + u;
+            if (s < n) {
+                if (((__double2hiint(d) >> 20) & 0x7ff) <= 723) d = -PIV;  // |d| < 2^-299
+                const double y = rcp_fast(d), l = al[u] * y;
+                if (live) {
+                    Y[(size_t)(half ? n - 1 - s : s) * ld + k] = y;
+                    if (s < n - 1) L[(size_t)(half ? n - 2 - s : s) * ld + k] = l;
+                }
+                d = fma(-al[u], l, -lam);
+            }
+        }
+    }
+}
+
+// argmin |gamma_i| over the rows (the lower on ties) and gamma there.
+__device__ __forceinline__ int twist_index(int n, const double* __restrict__ as, double lam, int half,
+                                           const double* Lp, const double* Lm, size_t ld, int k, double* gam) {
+    const int h = (n + 1) / 2, lo = half ? h : 0, hi = half ? n : h;
+    long long best = 0x7fffffffffffffffLL;
+    double bg = 0.0;
+    int br = lo;
+    for (int i0 = 0; i0 < h; i0 += TW_IB) {
+        double a[TW_IB], b[TW_IB], al[TW_IB + 1];
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const int i = min(lo + i0 + u, n - 1);
+            a[u] = i > 0 ? Lp[(size_t)(i - 1) * ld + k] : 0.0;
+            b[u] = i < n - 1 ? Lm[(size_t)i * ld + k] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u <= TW_IB; u++) {
+            const int e = min(lo + i0 + u, n - 1) - 1;
+            al[u] = e >= 0 ? as[min(e, n - 2)] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const double gm = fma(-al[u + 1], b[u], fma(-al[u], a[u], -lam));
+            const long long m = __double_as_longlong(gm) & 0x7fffffffffffffffLL;
+            if (lo + i0 + u < hi && m < best) {
+                best = m;
+                bg = gm;
+                br = lo + i0 + u;
+            }
+        }
+    }
+    const long long ob = __shfl_xor_sync(0xffffffffu, best, 16);
+    const double og = __shfl_xor_sync(0xffffffffu, bg, 16);
+    const int orow = __shfl_xor_sync(0xffffffffu, br, 16);
+    if (ob < best || (ob == best && orow < br)) {
+        bg = og;
+        br = orow;
+    }
+    *gam = bg;
+    return br;
+}
+
+// One step of inverse iteration with the factorisation twisted at r: on entry
+// Z holds b; afterwards gamma_r Y y of N y = b on this lane's side
+// (the forward part).  Returns y_r (both lanes).
+__device__ __forceinline__ double twist_forward(int n, int r, int half, double gam, const double* Y, const double* L,
+                                                double* Z, size_t ld, int k, bool live) {
+    double y = 0.0;
+    for (int s0 = 0; s0 < n - 1; s0 += TW_IB) {
+        double l[TW_IB], yi[TW_IB], zi[TW_IB];
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const int s = min(s0 + u, n - 2), row = half ? n - 1 - s : s;
+            zi[u] = Z[(size_t)row * ld + k];
+            yi[u] = Y[(size_t)row * ld + k];
+            l[u] = s > 0 ? L[(size_t)(half ? n - 1 - s : s - 1) * ld + k] : 0.0;  // edge to the previous row
+        }
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const int s = s0 + u, row = half ? n - 1 - s : s;
+            const bool act = s < n - 1 && (half ? row > r : row < r);
+            if (!__any_sync(0xffffffffu, act)) continue;
+            const double yn = fma(-l[u], y, zi[u]);
+            if (act) {
+                y = yn;
+                if (live) Z[(size_t)row * ld + k] = yn * (yi[u] * gam);
+            }
+        }
+    }
+    // this lane's share of y_r
+    const double br = Z[(size_t)r * ld + k];
+    const bool has = half ? r < n - 1 : r > 0;
+    const double mine = has ? L[(size_t)(half ? r : r - 1) * ld + k] * y : 0.0;
+    const double other = __shfl_xor_sync(0xffffffffu, mine, 16);
+    return half ? (br - other) - mine : (br - mine) - other;
+}
+
+// Z outwards from the twist index r with z_r = zr: z_i = (add ? Z_i : 0) -
+// l z_{previous}.  Returns |z|^2 and the sign of the entry of largest modulus
+// (the lowest on ties).
+__device__ __forceinline__ double twist_vector(int n, int r, double zr, bool add, int half, const double* L, double* Z,
+                                               size_t ld, int k, bool live, bool* neg) {
+    double z = zr, nrm = half ? 0.0 : zr * zr;
+    long long best = half ? -1 : (__double_as_longlong(zr) & 0x7fffffffffffffffLL);
+    int bi = r;
+    bool bneg = zr < 0.0;
+    if (live && !half) Z[(size_t)r * ld + k] = zr;
+    for (int s0 = 0; s0 < n - 1; s0 += TW_IB) {
+        double l[TW_IB], t[TW_IB];
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const int s = min(s0 + u, n - 2), e = half ? s : n - 2 - s;  // edge between rows e and e + 1
+            l[u] = L[(size_t)e * ld + k];
+            t[u] = add ? Z[(size_t)(half ? e + 1 : e) * ld + k] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < TW_IB; u++) {
+            const int e = half ? s0 + u : n - 2 - (s0 + u);
+            const bool act = s0 + u < n - 1 && (half ? e >= r : e < r);
+            if (!__any_sync(0xffffffffu, act)) continue;
+            const double zn = fma(-l[u], z, t[u]);
+            const double sq = fma(zn, zn, nrm);
+            if (act) {
+                z = zn;
+                nrm = sq;
+                const int row = half ? e + 1 : e;
+                if (live) Z[(size_t)row * ld + k] = z;
+                const long long m = __double_as_longlong(z) & 0x7fffffffffffffffLL;
+                if (m > best || (m == best && row < bi)) {
+                    best = m;
+                    bi = row;
+                    bneg = __double_as_longlong(z) < 0;
+                }
+            }
+        }
+    }
+    const long long ob = __shfl_xor_sync(0xffffffffu, best, 16);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, 16);
+    const int on = __shfl_xor_sync(0xffffffffu, (int)bneg, 16);
+    if (ob > best || (ob == best && oi < bi)) bneg = on != 0;
+    *neg = bneg;
+    // the same sum on both lanes of a pair
+    const double other = __shfl_xor_sync(0xffffffffu, nrm, 16);
+    return half ? other + nrm : nrm + other;
 }
 
 // Inverse iteration in double-float (about 2^-44 relative; Dekker's pair
