@@ -211,11 +211,11 @@ int skew_eig_host(int n, const double* A, int lda, int nev, double* lambda,
  * into device lambda[b], Z_re[b], Z_im[b] of leading dimension n[b]).  The
  * size arrays and the pointer arrays are host arrays; Z_re == Z_im == NULL
  * (the arrays) or Z_re[b] == Z_im[b] == NULL (one matrix) asks for
- * eigenvalues only.  Orders 2..1024 are solved together in one persistent
- * launch (see skew_batched_config below: each CTA takes whole matrices,
- * largest first, and runs unblocked Householder tridiagonalisation with the
- * matrix in shared or global memory, bisection, inverse iteration and the
- * back-transform), always in FP64; larger orders run the two-step solve of
+ * eigenvalues only.  Orders 2..1024 are solved together, stage by stage (see
+ * skew_batched_config below: unblocked Householder tridiagonalisation, one
+ * thread-block cluster or one CTA a matrix, largest first; then bisection,
+ * the tridiagonals' eigenvectors and the back-transform of all matrices in one
+ * launch each), always in FP64; larger orders run the two-step solve of
  * skew_eig_ex one after another in `opts`' mode.  Not in the paper (it solves one matrix per run).
  * Asynchronous on `stream`.  skew_eig_batched takes its workspace from the
  * library pool (stream-ordered, freed on the stream) and reports no per-matrix
@@ -236,15 +236,16 @@ int skew_eig_batched_ex(int count, const int* n, const double* const* A, const i
                         size_t ws_bytes, int* d_info, void* stream);
 
 /*
- * Batched solve as a plan: one persistent launch for the whole batch.
+ * Batched solve as a plan: about ten launches for the whole batch.
  * Not in the paper (it solves one matrix per run; each matrix here follows
  * Algorithm 1 in its one-step form: unblocked Householder tridiagonalisation,
  * Lemma-1 link, bisection and inverse iteration, D map and back
  * transformation, FP64 throughout).
  *
- * skew_batched_config sets the launch: ctas_per_sm (1..4) CTAs of 256 threads
- * per SM take matrices from a device work counter, largest first; orders up to
- * smem_max_n (0..160; capped by the shared memory of ctas_per_sm CTAs per SM)
+ * skew_batched_config sets the reduction of the orders up to 96: ctas_per_sm
+ * (1..4) CTAs of 256 threads per SM take matrices from a device work counter,
+ * largest first (larger orders take a thread-block cluster each, whose size the
+ * library chooses); orders up to smem_max_n (0..160; capped by the shared memory of ctas_per_sm CTAs per SM)
  * keep the working matrix in shared memory, larger ones in global memory.
  * skew_batched_set_config / get_config hold the process-wide default used by
  * skew_eig_batched(_ex) and by plans created with cfg == NULL (initially
@@ -257,7 +258,7 @@ int skew_eig_batched_ex(int count, const int* n, const double* const* A, const i
  * `stream` and synchronises it, and fixes the launch parameters.  The device
  * buffers named in the call must stay valid while the plan is used.
  * skew_batched_plan_exec then only clears d_info (may be NULL; per matrix 0 or
- * 1000 + j) and the work counter and launches the persistent kernel: no host
+ * 1000 + j) and the work counters and launches the stages: no host
  * synchronisation and no allocation, so the call can be captured into a CUDA
  * graph and replayed.  skew_batched_plan_tune times every candidate
  * configuration on the plan's batch (one warm-up and two timed runs each, CUDA

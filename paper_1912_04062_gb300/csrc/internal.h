@@ -222,8 +222,10 @@ void refine_stats_flush();
 void refine_stats_discard();
 
 // ---- batched.cu (many small independent solves) ------------------------------
-// Largest order of the one-CTA shared-memory path, and of the batched path
-// (one CTA per matrix, working matrix in global memory above the former).
+// Largest order reduced by one CTA (larger ones by a thread-block cluster: order
+// 160 takes 3.2 ms on one CTA and 0.4 ms on a cluster), bound of the
+// shared-memory threshold of skew_batched_config, largest order of the batched path.
+constexpr int BATCH_ONE_CTA = 96;
 constexpr int BATCH_SMALL_MAX = 160;
 constexpr int BATCH_MAX = 1024;
 struct BatchProblem {
@@ -233,15 +235,19 @@ struct BatchProblem {
     int* info;                   // device status word of this matrix (may be null)
 };
 size_t batched_small_ws(int count, const BatchProblem* probs);
-// every n in [2, BATCH_MAX]; FP64 throughout; one persistent launch with the
-// process-wide default configuration
+// every n in [2, BATCH_MAX]; FP64 throughout; the process-wide default
+// configuration
 int batched_small(cudaStream_t st, int count, const BatchProblem* probs, void* ws, size_t ws_bytes, int maxit);
-// The uploaded item table of a batch (device pointers into the workspace).
+// The uploaded tables of a batch (device pointers into the workspace).
 struct BatchPlanDev {
     const void* items;  // per-matrix descriptors (batched.cu's layout)
-    const int* order;   // matrices largest first
-    int* next;          // work counter of the persistent launch
-    int count, nmax;
+    const int* order;   // matrices largest first; the first nlarge take clusters
+    const void *bisect, *twist, *gram, *gsum, *wy;  // work units of the stages
+    void* clu;          // clusters of close eigenvalues
+    int* cnt;           // work counters of the two reductions, number of clusters
+    int nbisect, ntwist, ngram, ngsum, nwy;
+    int count, nlarge, nmax;
+    int cl_size, cl_count;  // the larger orders' clusters: CTAs each, how many
 };
 struct BatchLaunch {
     int ctas, grid;

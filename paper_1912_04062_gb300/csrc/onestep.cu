@@ -29,12 +29,15 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "onestep_dev.cuh"
 
 namespace sk {
+
+using namespace onestep;
+
 namespace {
 
 constexpr int OT = 256;     // threads of the reduction kernel
-constexpr int OW = OT / 32;
 constexpr int OMAXR = 64;   // rows of one CTA at most (n <= 64 G)
 
 struct OsArgs {
@@ -50,122 +53,10 @@ struct OsArgs {
     int srows;     // own rows kept in shared memory (the last ones: they live longest)
 };
 
-// Totals over the warp of N values per lane by exchanging halves: 5 levels,
-// about N additions instead of 5 N.  Afterwards a[0 .. cnt) of a lane are the
-// totals of the values first .. first + cnt - 1.
-template <int N>
-struct WarpSums {
-    static constexpr int H1 = (N + 1) / 2, H2 = (H1 + 1) / 2, H3 = (H2 + 1) / 2, H4 = (H3 + 1) / 2,
-                         H5 = (H4 + 1) / 2;
-    int first = 0, cnt = N;
-    template <int L, int H, int B>
-    SK_DEV void level(double (&a)[N], int lane) {
-        const bool up = lane & B;
-#pragma unroll
-        for (int i = 0; i < H; i++) {
-            const double hi = (i + H < L) ? a[i + H < N ? i + H : 0] : 0.0;
-            const double keep = up ? hi : a[i], send = up ? a[i] : hi;
-            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, B);
-        }
-        first += up ? H : 0;
-        cnt = up ? max(cnt - H, 0) : min(cnt, H);
-    }
-    SK_DEV void run(double (&a)[N], int lane) {
-        level<N, H1, 16>(a, lane);
-        level<H1, H2, 8>(a, lane);
-        level<H2, H3, 4>(a, lane);
-        level<H3, H4, 2>(a, lane);
-        level<H4, H5, 1>(a, lane);
-    }
-};
-
-// The rank-2 update of RC own rows (base, base + stride, ...; matrix rows i0,
-// i0 + G, ...) and their products with x, columns ja + 32 (warp + 4 t) + lane.
-// The row sums of this warp go to part[row * OCW].  GLB: rows in global
-// memory, the next step's elements are loaded ahead.
-constexpr int OCW = OW;  // warps of the pass
-
-template <int RC, bool GLB>
-SK_DEV void os_rows(double* base, size_t stride, int i0, int G, int n, int k, int ja, double sigma, const double* u,
-                    const double* p, const double* x, int warp, int lane, double* part) {
-    double ui[RC], pi[RC], acc[RC];
-#pragma unroll
-    for (int r = 0; r < RC; r++) {
-        ui[r] = sigma * u[i0 + r * G];
-        pi[r] = -sigma * p[i0 + r * G];
-        acc[r] = 0.0;
-    }
-    auto step = [&](int j, const double (&in)[RC]) {
-        const double uj = u[j], pj = p[j], xj = (j > k) ? x[j] : 0.0;
-        double a[RC];
-#pragma unroll
-        for (int r = 0; r < RC; r++) a[r] = fma(ui[r], pj, in[r]);
-#pragma unroll
-        for (int r = 0; r < RC; r++) {
-            a[r] = fma(pi[r], uj, a[r]);
-            if (j == i0 + r * G) a[r] = 0.0;
-            base[r * stride + j] = a[r];
-        }
-#pragma unroll
-        for (int r = 0; r < RC; r++) acc[r] = fma(a[r], xj, acc[r]);
-    };
-    int j = ja + 32 * warp + lane;
-    if (GLB) {
-        double nx[RC];
-#pragma unroll
-        for (int r = 0; r < RC; r++) nx[r] = j < n ? base[r * stride + j] : 0.0;
-#pragma unroll 1
-        for (; j < n; j += 32 * OCW) {
-            const int jn = j + 32 * OCW;
-            double in[RC];
-#pragma unroll
-            for (int r = 0; r < RC; r++) {
-                in[r] = nx[r];
-                nx[r] = jn < n ? base[r * stride + jn] : 0.0;
-            }
-            step(j, in);
-        }
-    } else {
-#pragma unroll 1
-        for (; j < n; j += 32 * OCW) {
-            double in[RC];
-#pragma unroll
-            for (int r = 0; r < RC; r++) in[r] = base[r * stride + j];
-            step(j, in);
-        }
-    }
-    WarpSums<RC> ws;
-    ws.run(acc, lane);
-#pragma unroll
-    for (int i = 0; i < WarpSums<RC>::H5; i++)
-        if (i < ws.cnt) part[(ws.first + i) * OCW] = acc[i];
-}
-
-template <bool GLB>
-SK_DEV void os_rows_any(int cnt, double* base, size_t stride, int i0, int G, int n, int k, int ja, double sigma,
-                        const double* u, const double* p, const double* x, int warp, int lane, double* part) {
-    while (cnt > 0) {
-        const int c = min(cnt, 8);
-        switch (c) {
-        case 1: os_rows<1, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
-        case 2: os_rows<2, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
-        case 3: os_rows<3, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
-        case 4: os_rows<4, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
-        case 5: os_rows<5, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
-        case 6: os_rows<6, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
-        case 7: os_rows<7, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part); break;
-        default: os_rows<8, GLB>(base, stride, i0, G, n, k, ja, sigma, u, p, x, warp, lane, part);
-        }
-        cnt -= c;
-        base += (size_t)c * stride;
-        i0 += c * G;
-        part += c * OCW;
-    }
-}
-
 __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
     extern __shared__ __align__(16) double os_sm[];
     __shared__ double s_part[OMAXR][OCW];
+    __shared__ double2 s_coef[OMAXR];  // sigma u_i, -sigma p_i of the own rows
     __shared__ double s_red[4];
     __shared__ double s_sc[4];  // beta, sigma, 1 / u_0, u_0
     __shared__ int s_ok;
@@ -214,23 +105,21 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
         // ---- 2. update the own rows i > k and multiply by x
         const int rf = (k + 1 > g) ? (k + 1 - g + G - 1) / G : 0;  // first own row below k
         const int R = Rt - rf;
-        const int ja = (k + 1) & ~3;
         const int rg = max(rs0, rf) - rf;  // rows of global memory
-        if (rg > 0)
-            os_rows_any<true>(rg, o.F + (size_t)(g + rf * G) * n, (size_t)G * n, g + rf * G, G, n, k, ja, sigma, u, p,
-                              x, warp, lane, &s_part[0][warp]);
-        os_rows_any<false>(R - rg, rows + (size_t)(rf + rg - rs0) * ldn, ldn, g + (rf + rg) * G, G, n, k, ja, sigma, u,
-                           p, x, warp, lane, &s_part[rg][warp]);
+        for (int r = t; r < R; r += OT)
+            s_coef[r] = make_double2(sigma * u[g + (rf + r) * G], -sigma * p[g + (rf + r) * G]);
+        __syncthreads();
+        const int nseg = R >= 32 ? 1 : R >= 16 ? 2 : R >= 8 ? 4 : 8;
+        os_pass<8>(nseg, R, rg, o.F + (size_t)(g + rf * G) * n, rows + (size_t)(rf + rg - rs0) * ldn, n, ldn, g + rf * G, G,
+                   k, s_coef, u, p, x, warp, lane, s_part);
         __syncthreads();
         if (warp == 0) {
             // ---- 3. publish the products and the next column, arrive, wait
             double2* out = o.qa + (size_t)((k + 1) & 1) * n;
             for (int r = lane; r < R; r += 32) {
                 const int i = g + (rf + r) * G;
-                const double* q = s_part[r];
                 const double* row = r >= rg ? rows + (size_t)(rf + r - rs0) * ldn : o.F + (size_t)i * n;
-                __stcg(out + i, make_double2(((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7])),
-                                             row[k + 1]));
+                __stcg(out + i, make_double2(os_row_sum(s_part[r], nseg), row[k + 1]));
             }
             __syncwarp();
             target += (unsigned)min(G, n - 1 - k);
@@ -329,210 +218,31 @@ os_full_kernel(int n, const double* __restrict__ A, int lda, double* __restrict_
     if (bad) sk_set_error(status, SKEW_ERR_NONFINITE);
 }
 
-// ---- back-transformation: Z <- H_0 H_1 ... H_{n-3} Z ------------------------
-// Panels of 64 reflectors (the last one padded with zero columns) act as one
-// compact WY block (Eq. 7).  T is not formed: T^-1 = diag(1 / tau) + the strict
-// upper triangle of V^T V, so T y is a back substitution with V^T V.
-
-constexpr int GR = 256;  // rows of one Gram partial
-constexpr int PB = 64;   // reflectors per panel
-
-// Upper triangle of V_p^T V_p over GR rows: CTA (p, s), 136 threads with one
-// 4 x 4 tile each.  part: [s][p][column][row].
 __global__ void __launch_bounds__(160)
 os_gram_kernel(int n, const double* __restrict__ V, int ldv, double* __restrict__ part) {
-    const int p = blockIdx.x, s = blockIdx.y, P = gridDim.x, t = threadIdx.x;
-    const int o = p * PB + 1, lo = o + s * GR, hi = min(n, lo + GR);
+    const int p = blockIdx.x, s = blockIdx.y, P = gridDim.x;
+    const int lo = p * PB + 1 + s * GR;
     if (lo >= n) return;
-    __shared__ double vs[PB][33];
-    int ti = 0, tj = 0;
-    if (t < 136) {
-        int e = t;  // tile (ti, tj), ti <= tj
-        while (e > tj) e -= ++tj;
-        ti = e;
-    }
-    double acc[4][4] = {};
-    for (int r0 = lo; r0 < hi; r0 += 32) {
-        for (int e = t; e < PB * 32; e += 160) {
-            const int r = e & 31, c = e >> 5;
-            vs[c][r] = (r0 + r < hi) ? V[(size_t)(p * PB + c) * ldv + r0 + r] : 0.0;
-        }
-        __syncthreads();
-        if (t < 136) {
-#pragma unroll 4
-            for (int r = 0; r < 32; r++) {
-                double a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; i++) a[i] = vs[4 * ti + i][r], b[i] = vs[4 * tj + i][r];
-#pragma unroll
-                for (int i = 0; i < 4; i++)
-#pragma unroll
-                    for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-            }
-        }
-        __syncthreads();
-    }
-    if (t < 136) {
-        double* q = part + ((size_t)s * P + p) * PB * PB;
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-#pragma unroll
-            for (int i = 0; i < 4; i++) q[(size_t)(4 * tj + j) * PB + 4 * ti + i] = acc[i][j];
-    }
+    os_gram_body(V + (size_t)p * PB * ldv, ldv, lo, min(n, lo + GR), part + ((size_t)s * P + p) * PB * PB);
 }
 
-// Sums the partials in order.  scaled: Gt[p][i][l] = (V^T V)_{l i} tau_i for
-// l < i, 0 elsewhere (the back substitution's rows); else the plain upper
-// triangle, mirrored.
 __global__ void __launch_bounds__(256)
 os_gram_sum_kernel(int n, const double* __restrict__ part, const double* __restrict__ tau, double* __restrict__ Gt,
                    int scaled) {
     const int p = blockIdx.x, P = gridDim.x;
     const int m = n - (p * PB + 1), S = (m + GR - 1) / GR;
-    for (int e = blockIdx.y * 256 + threadIdx.x; e < PB * PB; e += gridDim.y * 256) {
-        const int l = e % PB, i = e / PB;
-        double g = 0.0;
-        if (l < i || (!scaled && l == i))
-            for (int s = 0; s < S; s++) g += part[((size_t)s * P + p) * PB * PB + e];
-        if (scaled) {
-            Gt[(size_t)p * PB * PB + e] = g * tau[p * PB + i];
-        } else if (l <= i) {
-            Gt[(size_t)p * PB * PB + e] = g;
-            Gt[(size_t)p * PB * PB + (size_t)l * PB + i] = g;
-        }
-    }
+    os_gram_sum_body(part + (size_t)p * PB * PB, (size_t)P * PB * PB, S, tau + p * PB, Gt + (size_t)p * PB * PB, scaled,
+                     blockIdx.y * 256 + threadIdx.x, gridDim.y * 256);
 }
 
-constexpr int WT = 256;  // threads of the WY kernel
-
-// One CTA carries E eigenvectors (C = 2 E columns: real and imaginary parts)
-// through every panel without leaving the SM: the slab of Z stays in shared
-// memory, V streams from L2 (read twice per panel), and nothing is exchanged
-// between CTAs.  The D map is applied on the way in (Algorithm 1 step 3) and the parts
-// go straight to Z_re / Z_im.  Bound by the FP64 pipe: 2 FMA per element of
-// V and column.
 template <int E>
 __global__ void __launch_bounds__(WT, 1)
 os_wy_kernel(int n, int nev, const double* __restrict__ V, const double* __restrict__ Gt,
              const double* __restrict__ tau, const double* __restrict__ Qi, double* __restrict__ Zre,
              double* __restrict__ Zim, int ldz) {
-    constexpr int C = 2 * E, VG = C <= 8 ? 8 : 4, NP = 8 / VG;
-    constexpr int NW = WT / 32;
     extern __shared__ __align__(16) double wy_sm[];
-    double* ys = wy_sm;              // [64][C]
-    double* gs = ys + PB * C;        // [64][64]
-    double* zs = gs + PB * PB;       // [C][n]
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int e0 = blockIdx.x * E;
-    // D q: rows r mod 4 = 0, 1, 2, 3 of q are times 1, i, -1, -i
-    for (int i = t; i < n; i += WT) {
-#pragma unroll
-        for (int e = 0; e < E; e++) {
-            double q = e0 + e < nev ? Qi[(size_t)i * nev + e0 + e] : 0.0;
-            if (i & 2) q = -q;
-            zs[(size_t)(2 * e) * n + i] = (i & 1) ? 0.0 : q;
-            zs[(size_t)(2 * e + 1) * n + i] = (i & 1) ? q : 0.0;
-        }
-    }
-    const int P = (n - 2 + PB - 1) / PB;
-    for (int p = P - 1; p >= 0; p--) {
-        const int o = p * PB + 1;
-        const double* Vp = V + (size_t)p * PB * n;
-        for (int e = t; e < PB * PB; e += WT) gs[e] = Gt[(size_t)p * PB * PB + e];
-        __syncthreads();
-        // Y = V_p^T Z: a warp takes 8 columns of V, lanes the rows
-#pragma unroll 1
-        for (int pass = 0; pass < NP; pass++) {
-            const int v0 = warp * 8 + pass * VG;
-            const double* Vc = Vp + (size_t)v0 * n;
-            double acc[VG * C];
-#pragma unroll
-            for (int i = 0; i < VG * C; i++) acc[i] = 0.0;
-            double vv[VG], vn[VG];
-            int r = o + lane;
-#pragma unroll
-            for (int i = 0; i < VG; i++) vn[i] = r < n ? Vc[(size_t)i * n + r] : 0.0;
-            for (; r - lane < n; r += 32) {
-#pragma unroll
-                for (int i = 0; i < VG; i++) {
-                    vv[i] = vn[i];
-                    vn[i] = r + 32 < n ? Vc[(size_t)i * n + r + 32] : 0.0;
-                }
-                const int rr = r < n ? r : n - 1;
-#pragma unroll
-                for (int c = 0; c < C; c++) {
-                    const double z = zs[(size_t)c * n + rr];
-#pragma unroll
-                    for (int i = 0; i < VG; i++) acc[i * C + c] = fma(vv[i], z, acc[i * C + c]);
-                }
-            }
-            WarpSums<VG * C> ws;
-            ws.run(acc, lane);
-#pragma unroll
-            for (int i = 0; i < WarpSums<VG * C>::H5; i++)
-                if (i < ws.cnt) ys[v0 * C + ws.first + i] = acc[i];
-        }
-        __syncthreads();
-        // y <- T y by back substitution, one warp per column
-        for (int c = warp; c < C; c += NW) {
-            double y0 = ys[lane * C + c], y1 = ys[(lane + 32) * C + c];
-#pragma unroll 4
-            for (int i = 63; i >= 32; i--) {
-                const double b = __shfl_sync(0xffffffffu, y1, i - 32);
-                y1 = fma(-gs[i * PB + lane + 32], b, y1);
-                y0 = fma(-gs[i * PB + lane], b, y0);
-            }
-#pragma unroll 4
-            for (int i = 31; i > 0; i--) {
-                const double b = __shfl_sync(0xffffffffu, y0, i);
-                y0 = fma(-gs[i * PB + lane], b, y0);
-            }
-            ys[lane * C + c] = -tau[p * PB + lane] * y0;
-            ys[(lane + 32) * C + c] = -tau[p * PB + lane + 32] * y1;
-        }
-        __syncthreads();
-        // Z -= V_p y: warps take blocks of 32 rows
-        for (int rb = warp; o + 32 * rb < n; rb += NW) {
-            const int r = o + 32 * rb + lane, rr = r < n ? r : n - 1;
-            double z[C];
-#pragma unroll
-            for (int c = 0; c < C; c++) z[c] = zs[(size_t)c * n + rr];
-            const double* Vr = Vp + rr;
-            double vn[8];
-#pragma unroll
-            for (int i = 0; i < 8; i++) vn[i] = Vr[(size_t)i * n];
-            for (int v = 0; v < PB; v += 8) {
-                double vv[8];
-                const int nx = v + 8 < PB ? v + 8 : v;
-#pragma unroll
-                for (int i = 0; i < 8; i++) {
-                    vv[i] = vn[i];
-                    vn[i] = Vr[(size_t)(nx + i) * n];
-                }
-#pragma unroll
-                for (int i = 0; i < 8; i++)
-#pragma unroll
-                    for (int c = 0; c < C; c += 2) {
-                        const double2 y = *reinterpret_cast<const double2*>(ys + (v + i) * C + c);
-                        z[c] = fma(vv[i], y.x, z[c]);
-                        z[c + 1] = fma(vv[i], y.y, z[c + 1]);
-                    }
-            }
-            if (r < n) {
-#pragma unroll
-                for (int c = 0; c < C; c++) zs[(size_t)c * n + r] = z[c];
-            }
-        }
-        __syncthreads();
-    }
-    for (int e = 0; e < E && e0 + e < nev; e++)
-        for (int i = t; i < n; i += WT) {
-            Zre[(size_t)(e0 + e) * ldz + i] = zs[(size_t)(2 * e) * n + i];
-            Zim[(size_t)(e0 + e) * ldz + i] = zs[(size_t)(2 * e + 1) * n + i];
-        }
+    os_wy_body<E>(n, nev, blockIdx.x * E, V, Gt, tau, Qi, Zre, Zim, ldz, wy_sm);
 }
-
-size_t wy_smem(int n, int E) { return sizeof(double) * ((size_t)PB * 2 * E + PB * PB + 2 * (size_t)E * n); }
 
 template <int E>
 cudaError_t wy_launch(cudaStream_t st, int n, int nev, const double* V, const double* Gt, const double* tau,
@@ -548,7 +258,7 @@ cudaError_t wy_launch(cudaStream_t st, int n, int nev, const double* V, const do
 int os_srows(int n, int G) {
     const int rmax = (n + G - 1) / G;
     const size_t vec = 3 * sizeof(double) * (size_t)(n | 1), row = sizeof(double) * (size_t)(n | 1);
-    const size_t cap = 222 * 1024;  // of 227 KB: the static arrays take about 4.3 KB
+    const size_t cap = 221 * 1024;  // of 227 KB: the static arrays take about 5.3 KB
     const int fit = vec + row > cap ? 0 : (int)((cap - vec) / row);
     return std::min(rmax, fit);
 }

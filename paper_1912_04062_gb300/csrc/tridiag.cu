@@ -130,65 +130,17 @@ __device__ __forceinline__ int sturm_df(int n, const float* __restrict__ a2s, co
     return cnt;
 }
 
-// FP32 Sturm count of the scaled matrix S / g at x (|x| ~ 1): the recurrence
-// of sturm() with pivots below FLT_MIN raised to FLT_MIN.
-__device__ __forceinline__ int sturm32(int n, const float* __restrict__ a2s, float x) {
-    int cnt = 0;
-    float d = -x;
-    if (fabsf(d) < FLT_MIN) d = -FLT_MIN;
-    cnt += (d < 0.f);
-    for (int i = 1; i < n; i++) {
-        d = -x - __fdividef(a2s[i - 1], d);
-        if (fabsf(d) < FLT_MIN) d = -FLT_MIN;
-        cnt += (d < 0.f);
-    }
-    return cnt;
-}
-
-// Bracketing pass in FP32 (64 times the FP64 rate on this part): L lanes
-// per wanted eigenvalue multisect [-1, 1] for S / g down to 8 eps32.  A
-// floating-point Sturm count is the exact count of a matrix whose entries are
-// perturbed by a few units of roundoff (Kahan), so lambda_j lies within a few
-// eps32 g of the FP32 bracket; the FP64 pass widens it by FP32_SLACK eps32 g
-// and checks it with FP64 counts before trusting it.
 template <int L>
-__device__ __forceinline__ unsigned lane_group(int lane) {
-    return L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << (lane & ~(L - 1));
-}
-
-template <int L>
-__global__ void bisect32_kernel(int n, int nev, const float* __restrict__ a2s, const TriScalars* sc,
-                                double* __restrict__ lohi) {
+__global__ void bisect32_kernel(int n, int nev, const float* __restrict__ a2s, double* __restrict__ lohi) {
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = gt / L, q = gt % L, lane = threadIdx.x & 31;
-    if (k >= nev) return;
-    const unsigned gmask = lane_group<L>(lane);
-    const int j = n - 1 - k;
-    float lo = -1.0f - 4.0f * FLT_EPSILON, hi = 1.0f + 4.0f * FLT_EPSILON;
-    for (int it = 0; it < 64; it++) {
-        const float w = hi - lo;
-        if (w <= 8.0f * FLT_EPSILON) break;
-        const float step = w * (1.0f / (L + 1));
-        const float x = lo + (float)(q + 1) * step;
-        const bool le = (x > lo && x < hi) ? (sturm32(n, a2s, x) <= j) : (x <= lo);
-        const int nle = __popc(__ballot_sync(gmask, le) & gmask);
-        const float nlo = (nle > 0) ? lo + (float)nle * step : lo;
-        const float nhi = (nle < L) ? lo + (float)(nle + 1) * step : hi;
-        if (!(nlo > lo || nhi < hi)) break;
-        lo = nlo;
-        hi = (nhi < hi) ? nhi : hi;
-    }
-    if (q == 0) {
-        lohi[2 * k] = (double)lo;  // in units of g
-        lohi[2 * k + 1] = (double)hi;
-    }
+    const int k = gt / L;
+    if (k < nev) bisect32_body<L>(n, k, gt % L, threadIdx.x & 31, a2s, lohi);
 }
 
 // Second pass: L lanes multisect the FP32 bracket (widened by FP32_SLACK
 // eps32, checked with double-float counts and widened eightfold until the
 // check holds) with double-float counts down to DF_WIDTH.  Writes the
 // bracket (units of g) back and, in lambda, its midpoint times g.
-constexpr double FP32_SLACK = 64.0;
 constexpr double DF_WIDTH = 1.0 / 4398046511104.0;  // 2^-42
 template <int L>
 __global__ void bisect_df_kernel(int n, int nev, const float* __restrict__ a2s, const float* __restrict__ a2l,
@@ -295,69 +247,15 @@ __global__ void bisect_kernel(int n, int nev, const double* __restrict__ a2, con
     if (q == 0) lambda[k] = lo + 0.5 * (hi - lo);
 }
 
-// FP64 multisection on the zero-diagonal form (B B^T at x^2, m = ceil(n/2)
-// steps; the wanted eigenvalues are >= 0, so the search stays in [0, g]),
-// straight from the FP32 bracket.  The first step's points span the bracket
-// widened by FP32_SLACK eps32 g; an eigenvalue outside them leaves the interval
-// to the end of [0, g] on that side, so the bracket need not be trusted.
-// Bound by the FP64 instructions of one chain (6 x 64 clocks a step when a
-// scheduler has one warp), so L is the largest power of two that still gives
-// every warp a scheduler of its own: 12 three-section steps from a
-// double-float bracket took 3.3 ms at n = 500, nev = 250 with the passes
-// before it.
 template <int L>
 __global__ void __launch_bounds__(64) bisect_bd_kernel(int n, int nev, const TriScalars* sc,
                                                        const double* __restrict__ lohi, double* __restrict__ lambda,
                                                        const double* __restrict__ a2e,
                                                        const double* __restrict__ b2e) {
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = gt / L, q = gt % L, lane = threadIdx.x & 31;
-    if (k >= nev) return;
-    const unsigned gmask = lane_group<L>(lane);
-    const int m = (n + 1) / 2, j = m - 1 - k;
-    if (n == 1 || sc->g == 0.0) {
-        if (q == 0) lambda[k] = 0.0;
-        return;
-    }
-    const double gs = sc->g * sc->down;  // in [1, 2)
-    const double ghi = gs + 2.0 * DBL_EPSILON * gs;
-    const double slack = FP32_SLACK * FLT_EPSILON * gs;
-    double lo = 0.0, hi = ghi;
-    // the first points: a, ..., b inclusive
-    double a = fmax(0.0, lohi[2 * k] * gs - slack), step = (fmin(ghi, lohi[2 * k + 1] * gs + slack) - a) / (double)(L - 1);
-    bool first = true;
-    for (int it = 0; it < 4000; it++) {
-        const double w = hi - lo;
-        const double tol = 2.0 * DBL_EPSILON * hi + 1e-300;
-        if (!(w > tol)) break;
-        if (!first) {
-            step = w / (double)(L + 1);
-            a = lo + step;
-        }
-        const double x = a + (double)q * step;
-        const bool le = (x > lo && x < hi) ? (bd_count_scaled(m, a2e, b2e, x * x) <= j) : (x <= lo);
-        const int nle = __popc(__ballot_sync(gmask, le) & gmask);
-        const double nlo = (nle > 0) ? fmax(lo, a + (double)(nle - 1) * step) : lo;
-        const double nhi = (nle < L) ? fmin(hi, a + (double)nle * step) : hi;
-        if (!first && !(nlo > lo || nhi < hi)) break;
-        first = false;
-        lo = nlo;
-        hi = nhi;
-    }
-    if (q == 0) lambda[k] = (lo + 0.5 * (hi - lo)) * sc->up;
+    const int k = gt / L;
+    if (k < nev) bisect_bd_body<L>(n, k, gt % L, threadIdx.x & 31, sc, lohi, lambda, a2e, b2e);
 }
-
-// ---- lockstep inverse iteration of clusters ---------------------------------
-// A cluster (two or more eigenvalues closer than ctol) is iterated in lockstep
-// rather than by one thread: in every iteration each member solves with its
-// own LU on its own thread, then the cluster's CTA orthogonalises the members
-// in index order (modified Gram-Schmidt, parallel over the rows), normalises
-// them and applies the growth test to each; the cluster stops one iteration
-// after all its members passed.  The vectors are an orthonormal basis of the
-// same invariant subspace, and the critical path is one member's solves
-// instead of the whole cluster's (16 x at the 1e-10 clusters of a clustered
-// spectrum).  Singletons keep the one-thread path.
-constexpr int CLU_T = 256;
 
 __global__ void clu_list_kernel(int nev, const double* __restrict__ lambda, const TriScalars* sc, double ctol_rel,
                                 int2* __restrict__ list, int* __restrict__ count) {
@@ -376,188 +274,14 @@ __global__ void clu_list_kernel(int nev, const double* __restrict__ lambda, cons
     if (threadIdx.x == 0) *count = c;
 }
 
-// Clusters come in two kinds.  Where all neighbouring gaps exceed TIGHT g each
-// member's own vector (twist_kernel) is accurate to about eps / TIGHT, and
-// one modified Gram-Schmidt pass orthogonalises the members: the overlaps it
-// removes are eps g / gap, which moves a residual by eps g only.  Tight
-// clusters (or ones with a member that failed the residual test, need[2 k] !=
-// 0) go through the lockstep iteration.
-constexpr double TIGHT = 1e-9;
-
-__device__ __forceinline__ bool clu_tight(const double* lambda, const double* need, double g, int k0, int m) {
-    for (int j = 0; j < m; j++)
-        if (need[2 * (k0 + j)] != 0.0 || (j + 1 < m && !(lambda[k0 + j] - lambda[k0 + j + 1] > TIGHT * g))) return true;
-    return false;
-}
-
-// Row of the largest abs(x_i) (the lowest on ties), CTA-wide.
-template <class F>
-__device__ __forceinline__ int block_argmax(int n, F absval, double* rv, int* ri) {
-    double best = -1.0;
-    int bi = 0x7fffffff;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double a = absval(i);
-        if (a > best) {
-            best = a;
-            bi = i;
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) {
-            best = ob;
-            bi = oi;
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    __syncthreads();
-    if (lane == 0) {
-        rv[warp] = best;
-        ri[warp] = bi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < nw; w++)
-            if (rv[w] > rv[0] || (rv[w] == rv[0] && ri[w] < ri[0])) {
-                rv[0] = rv[w];
-                ri[0] = ri[w];
-            }
-    }
-    __syncthreads();
-    const int r = ri[0];
-    __syncthreads();
-    return r < n ? r : 0;
-}
-
-// The Gram-Schmidt pass of a loose cluster: members in index order, each
-// normalised, its largest-modulus entry positive.
-__device__ void clu_mgs(int n, size_t ld, double* Q, int k0, int m, double* red, int* redi) {
-    const int t = threadIdx.x, T = blockDim.x;
-    for (int j = 0; j < m; j++) {
-        double* qj = Q + k0 + j;
-        for (int p = 0; p < j; p++) {
-            const double* qp = Q + k0 + p;
-            double d = 0.0;
-            for (int i = t; i < n; i += T) d = fma(qp[i * ld], qj[i * ld], d);
-            d = sk_block_sum(d, red);
-            for (int i = t; i < n; i += T) qj[i * ld] = fma(-d, qp[i * ld], qj[i * ld]);
-            __syncthreads();
-        }
-        double s = 0.0;
-        for (int i = t; i < n; i += T) s = fma(qj[i * ld], qj[i * ld], s);
-        s = sk_block_sum(s, red);
-        const int imax = block_argmax(n, [&](int i) { return fabs(qj[i * ld]); }, red, redi);
-        const double f = (qj[imax * ld] < 0.0 ? -1.0 : 1.0) / sqrt(s);
-        __syncthreads();
-        for (int i = t; i < n; i += T) qj[i * ld] *= f;
-        __syncthreads();
-    }
-}
-
-// Decision after an iteration: state 0 iterating, 1 all members passed (one
-// more iteration), 2 done.  ff = first member that failed the growth test
-// (m if none), bad = a member's norm was zero or not finite.
-__device__ __forceinline__ int clu_next_state(int st, int ff, int m, int bad, int it, int maxit, bool& fin,
-                                              bool& failed) {
-    int nst = (st == 1) ? 2 : (ff == m ? 1 : 0);
-    if (bad) nst = 0;
-    fin = bad || nst == 2 || it == maxit - 1;
-    failed = fin && nst == 0;
-    return nst;
-}
-
 __global__ void __launch_bounds__(CLU_T)
 invit_clu_kernel(int n, int nev, const double* __restrict__ alpha, const double* __restrict__ lambda,
-                 const TriScalars* sc, int maxit, InvitBufs bf, double* Q,
-                 const int2* __restrict__ list, const int* __restrict__ count, const double* __restrict__ need,
-                 int* __restrict__ fail) {
-    __shared__ double red[32];
-    __shared__ int redi[32];
-    __shared__ int s_ff, s_bad;
+                 const TriScalars* sc, int maxit, InvitBufs bf, double* Q, const int2* __restrict__ list,
+                 const int* __restrict__ count, const double* __restrict__ need, int* __restrict__ fail) {
     const int nc = *count;
-    const double g = sc->g;
-    const size_t ld = (size_t)nev;
-    const double eps = DBL_EPSILON, ptol = eps * g;
-    const double grow = 1.0 / (100.0 * sqrt((double)n) * eps * g);
-    const int t = threadIdx.x, T = blockDim.x;
     for (int b = blockIdx.x; b < nc; b += gridDim.x) {
-        const int2 cl = list[b];
-        const int k0 = cl.x, m = cl.y;
-        if (n == 1 || g == 0.0) {
-            for (int e = t; e < m * n; e += T) {
-                const int j = e / n, i = e % n;
-                Q[i * ld + k0 + j] = (i == k0 + j) ? 1.0 : 0.0;
-            }
-            continue;
-        }
-        if (!clu_tight(lambda, need, g, k0, m)) {
-            clu_mgs(n, ld, Q, k0, m, red, redi);
-            continue;
-        }
-        // the cluster's iterations one after another; st (clu_next_state) is
-        // the same in every thread
-        int st = 0;
-        for (int it = 0; it < maxit && st != 2; it++) {
-            // the members' solves, one thread each
-            for (int j = t; j < m; j += T) {
-                const int k = k0 + j;
-                if (it == 0) {
-                    invit_lu(n, alpha, lambda[k], ptol, bf, ld, k);
-                    invit_start(n, Q, ld, k);
-                }
-                invit_solve(n, bf, Q, ld, k);
-            }
-            if (t == 0) {
-                s_ff = m;
-                s_bad = 0;
-            }
-            __syncthreads();
-            // modified Gram-Schmidt in index order, normalisation, growth test
-            for (int j = 0; j < m; j++) {
-                double* qj = Q + k0 + j;
-                for (int p = 0; p < j; p++) {
-                    const double* qp = Q + k0 + p;
-                    double d = 0.0;
-                    for (int i = t; i < n; i += T) d = fma(qp[i * ld], qj[i * ld], d);
-                    d = sk_block_sum(d, red);
-                    for (int i = t; i < n; i += T) qj[i * ld] = fma(-d, qp[i * ld], qj[i * ld]);
-                    __syncthreads();
-                }
-                double s = 0.0;
-                for (int i = t; i < n; i += T) s = fma(qj[i * ld], qj[i * ld], s);
-                const double nrm = sqrt(sk_block_sum(s, red));
-                if (!(nrm > 0.0) || !isfinite(nrm)) {
-                    if (t == 0) {
-                        s_bad = 1;
-                        s_ff = min(s_ff, j);
-                    }
-                } else {
-                    const double inv = 1.0 / nrm;
-                    for (int i = t; i < n; i += T) qj[i * ld] *= inv;
-                    if (t == 0 && !(nrm >= grow)) s_ff = min(s_ff, j);
-                }
-                __syncthreads();
-            }
-            bool fin, failed;
-            const int nst = clu_next_state(st, s_ff, m, s_bad, it, maxit, fin, failed);
-            if (failed && t == 0) atomicMin(fail, k0 + s_ff);
-            if (fin) {
-                // largest-modulus entry of each vector positive (lowest index on ties)
-                for (int j = 0; j < m; j++) {
-                    double* qj = Q + k0 + j;
-                    const int imax = block_argmax(n, [&](int i) { return fabs(qj[i * ld]); }, red, redi);
-                    const bool neg = qj[imax * ld] < 0.0;  // read by all before any flip
-                    __syncthreads();
-                    if (neg)
-                        for (int i = t; i < n; i += T) qj[i * ld] = -qj[i * ld];
-                    __syncthreads();
-                }
-            }
-            st = fin ? 2 : nst;
-            __syncthreads();
-        }
+        __syncthreads();  // the previous cluster is done with shared memory
+        clu_body(n, nev, list[b].x, list[b].y, alpha, lambda, sc->g, maxit, bf, Q, need, fail);
     }
 }
 
@@ -686,76 +410,12 @@ invit_clu_df_kernel(int n, int nev, const float* __restrict__ alh, const float* 
     }
 }
 
-// Vectors of the eigenvalues that are alone within ctol, and of the members
-// of loose clusters.  polish: eigenvalues
-// accurate to rounding; the twisted vector is followed by one step of inverse
-// iteration with the same factorisation, which removes the share of the
-// neighbours that the rounding of lambda leaves in it (orthogonality 3.2 n eps
-// without it and 0.3 with it at n = 1001).  Otherwise eigenvalues known to
-// 2^-42 g: a second factorisation at the Rayleigh quotient of the first one's
-// vector (the caller refines).  A vector whose residual is above 100 sqrt(n)
-// eps g (the growth test of inverse iteration) is handed to the pivoted
-// inverse iteration.  About 14 FP64 instructions a row and vector, one warp a scheduler.
 __global__ void __launch_bounds__(32)
 twist_kernel(int n, int nev, const double* __restrict__ as, const double* __restrict__ alpha,
              const double* __restrict__ lambda, const TriScalars* sc, double ctol_rel, int maxit, int polish,
              InvitBufs bf, double* Q, double* __restrict__ need, int* __restrict__ fail) {
-    const int lane = threadIdx.x, half = lane >> 4;
-    const int kk = blockIdx.x * 16 + (lane & 15), k = min(kk, nev - 1);
-    const double g = sc->g, ctol = ctol_rel * g;
-    const size_t ld = (size_t)nev;
-    const bool single = starts_cluster(lambda, k, ctol) && (k + 1 >= nev || starts_cluster(lambda, k + 1, ctol));
-    const double tight = TIGHT * g;
-    const bool live = kk < nev && (single || (starts_cluster(lambda, k, tight) &&
-                                              (k + 1 >= nev || starts_cluster(lambda, k + 1, tight))));
-    if (kk < nev && !half) need[2 * k] = live ? 0.0 : 1.0;
-    if (!__any_sync(0xffffffffu, live)) return;
-    if (n == 1 || g == 0.0) {
-        if (live && !half)
-            for (int i = 0; i < n; i++) Q[i * ld + k] = (i == k) ? 1.0 : 0.0;
-        return;
-    }
-    double* Y = half ? bf.u1 : bf.u0;
-    double* L = half ? bf.ml : bf.u2;
-    double lam = lambda[k] * sc->down, gam = 0.0;
-    bool neg = false;
-    twist_factor(n, as, lam, half, Y, L, ld, k, live);
-    __syncwarp();
-    int r = twist_index(n, as, lam, half, bf.u2, bf.ml, ld, k, &gam);
-    double nrm = twist_vector(n, r, 1.0, false, half, L, Q, ld, k, live, &neg), res;
-    __syncwarp();
-    if (polish) {
-        const double n0 = nrm, yr = twist_forward(n, r, half, gam, Y, L, Q, ld, k, live);
-        __syncwarp();
-        nrm = twist_vector(n, r, yr, true, half, L, Q, ld, k, live, &neg);
-        res = fabs(gam) * sqrt(n0 / nrm);
-    } else {
-        const double dl = gam / nrm;
-        if (fabs(dl) < 1e-9) lam += dl;
-        twist_factor(n, as, lam, half, Y, L, ld, k, live);
-        __syncwarp();
-        r = twist_index(n, as, lam, half, bf.u2, bf.ml, ld, k, &gam);
-        nrm = twist_vector(n, r, 1.0, false, half, L, Q, ld, k, live, &neg);
-        res = fabs(gam) / sqrt(nrm);
-    }
-    const double inv = (neg ? -1.0 : 1.0) / sqrt(nrm);
-    const double gs = g * sc->down;
-    const bool ok = maxit > 0 && isfinite(inv) && res <= 100.0 * sqrt((double)n) * DBL_EPSILON * gs;
-    __syncwarp();
-    const int h = (n + 1) / 2, lo = half ? h : 0, hi = half ? n : h;
-    if (live && ok) {
-        for (int i0 = lo; i0 < hi; i0 += TW_IB) {
-            double z[TW_IB];
-#pragma unroll
-            for (int u = 0; u < TW_IB; u++)
-                if (i0 + u < hi) z[u] = Q[(size_t)(i0 + u) * ld + k];
-#pragma unroll
-            for (int u = 0; u < TW_IB; u++)
-                if (i0 + u < hi) Q[(size_t)(i0 + u) * ld + k] = z[u] * inv;
-        }
-    }
-    if (live && !ok && !half) need[2 * k] = 1.0;
-    if (live && !ok && !half && single) invit_cluster(n, nev, alpha, lambda, g, ctol_rel, maxit, bf, Q, fail, k, true);
+    twist_body(n, nev, blockIdx.x * 16, threadIdx.x, as, alpha, lambda, sc, ctol_rel, maxit, polish, bf, Q, need,
+               fail);
 }
 
 __global__ void invit_status_kernel(const int* fail, int nev, int* status) {
@@ -866,9 +526,9 @@ int tridiag_eig(cudaStream_t st, int n, const double* alpha, int nev, double* la
         // eight warps a scheduler, four beyond that
         const bool wide = nev <= sms * 32;
         if (wide)
-            bisect32_kernel<32><<<(32 * nev + 127) / 128, 128, 0, st>>>(n, nev, w.a2s, w.sc, w.lohi);
+            bisect32_kernel<32><<<(32 * nev + 127) / 128, 128, 0, st>>>(n, nev, w.a2s, w.lohi);
         else
-            bisect32_kernel<4><<<(4 * nev + 127) / 128, 128, 0, st>>>(n, nev, w.a2s, w.sc, w.lohi);
+            bisect32_kernel<4><<<(4 * nev + 127) / 128, 128, 0, st>>>(n, nev, w.a2s, w.lohi);
         count_launch();
         if (fp64 && !full) {
             // FP64 finish on the zero-diagonal form (half-length counts)

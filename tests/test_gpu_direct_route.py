@@ -94,3 +94,27 @@ def test_twisted_vectors_of_glued_blocks(n, glue):
     scale = float(lam[0])
     assert float((S @ Q - Q * lam).norm(dim=0).max()) <= 50 * n * EPS * scale
     assert float((Q.T @ Q - torch.eye(nev, device="cuda", dtype=Q.dtype)).norm()) <= 50 * n * EPS
+
+
+def test_batch_results_do_not_depend_on_the_cluster_size():
+    # orders around the one-CTA limit, around the changes of the pass's column
+    # split (72, 144 and 288 rows left) and around shared memory; alone (large
+    # clusters) and in a long batch (small ones) they give the same bits
+    import torch
+    import paper_1912_04062_gb300 as sk
+    sizes = [96, 97, 98, 145, 146, 289, 290, 500, 777, 1024]
+    mats = [sk.fortran(torch.from_numpy(inputs.random_skew(n, seed=7300 + n)).cuda()) for n in sizes]
+    nevs = [n // 2 if n != 500 else 33 for n in sizes]
+    lam, Zr, Zi, info = sk.skew_eig_batched(mats * 12, nevs * 12, info=True)
+    torch.cuda.synchronize()
+    assert int(info.abs().max()) == 0
+    for i, (A, nev) in enumerate(zip(mats, nevs)):
+        l1, zr1, zi1 = (v[0] for v in sk.skew_eig_batched([A], [nev]))
+        torch.cuda.synchronize()
+        for j in (i, i + 11 * len(sizes)):
+            assert torch.equal(l1, lam[j]) and torch.equal(zr1, Zr[j]) and torch.equal(zi1, Zi[j])
+        n = A.shape[0]
+        r, o, f = sk.metrics(A, l1, zr1, zi1)
+        assert r <= 50 * n * EPS * f and o <= 50 * n * EPS
+        ref, _, _ = _solve(A, nev, sk.Options(), vectors=False)
+        assert float((ref - l1).abs().max()) <= 1e-12 * float(ref[0])
