@@ -306,7 +306,7 @@ cluster_reduce_kernel(const BItem* __restrict__ items, const int* __restrict__ o
                 for (int r = t; r < R; r += 256)
                     s_coef[r] = make_double2(sigma * u[g + (rf + r) * G], -sigma * p[g + (rf + r) * G]);
                 asm volatile("bar.sync 1, 256;" ::: "memory");
-                os_pass<4>(nseg, R, rg, it.S + (size_t)(g + rf * G) * n, rows + (size_t)(rf + rg - rs0) * ldn, n, ldn,
+                os_pass<4>(nseg, nseg, R, rg, it.S + (size_t)(g + rf * G) * n, rows + (size_t)(rf + rg - rs0) * ldn, n, ldn,
                            g + rf * G, G, k, s_coef, u, p, x, warp, lane, s_part);
                 asm volatile("bar.sync 1, 256;" ::: "memory");
                 // publish (q_i, a_i) of the own rows to every CTA

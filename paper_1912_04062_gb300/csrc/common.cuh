@@ -43,7 +43,6 @@ SK_DEV unsigned sk_atom_add_release(unsigned* p, unsigned v) {
     asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
 }
-
 // Grid-wide barrier for cooperative launches (all CTAs co-resident).  The
 // counter grows monotonically; the caller tracks its own epoch.  Returns false
 // (and records SKEW_ERR_DEVICE_TIMEOUT) when the wait cap (polls) is reached or

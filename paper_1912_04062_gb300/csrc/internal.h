@@ -73,6 +73,14 @@ cudaError_t onestep_full(cudaStream_t st, int n, const double* A, int lda, doubl
 // as in band_reduce.
 int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, double* alpha, void* ws,
                    size_t ws_bytes, int* d_status, unsigned spin_cap);
+// The same in double-float (onestep_df.cu) for a caller that refines the
+// result: F holds pairs of floats (8 bytes an element); ws is shared by the two
+// calls (onestep_ws bytes) and carries the scaling from one to the other.
+int onestep_df_max();
+int onestep_df_full(cudaStream_t st, int n, const double* A, int lda, void* F, int check, void* ws, size_t ws_bytes,
+                    int* status);
+int onestep_df_reduce(cudaStream_t st, int n, void* F, double* V, double* tau, double* alpha, void* ws,
+                      size_t ws_bytes, int* d_status, unsigned spin_cap);
 // FP64 Z = H_0 H_1 ... H_{n-3} D Q from the interleaved tridiagonal vectors Qi
 // (Qi[i * nev + k]), for the sizes of onestep_wy_fits.
 bool onestep_wy_fits(int n, int nev);

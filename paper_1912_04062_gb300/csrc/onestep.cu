@@ -109,8 +109,8 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
         for (int r = t; r < R; r += OT)
             s_coef[r] = make_double2(sigma * u[g + (rf + r) * G], -sigma * p[g + (rf + r) * G]);
         __syncthreads();
-        const int nseg = R >= 32 ? 1 : R >= 16 ? 2 : R >= 8 ? 4 : 8;
-        os_pass<8>(nseg, R, rg, o.F + (size_t)(g + rf * G) * n, rows + (size_t)(rf + rg - rs0) * ldn, n, ldn, g + rf * G, G,
+        const int nss = R - rg >= 16 ? 1 : R - rg >= 8 ? 2 : R - rg >= 4 ? 4 : 8, nsg = rg >= 16 ? 4 : 8;
+        os_pass<8>(nsg, nss, R, rg, o.F + (size_t)(g + rf * G) * n, rows + (size_t)(rf + rg - rs0) * ldn, n, ldn, g + rf * G, G,
                    k, s_coef, u, p, x, warp, lane, s_part);
         __syncthreads();
         if (warp == 0) {
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
             for (int r = lane; r < R; r += 32) {
                 const int i = g + (rf + r) * G;
                 const double* row = r >= rg ? rows + (size_t)(rf + r - rs0) * ldn : o.F + (size_t)i * n;
-                __stcg(out + i, make_double2(os_row_sum(s_part[r], nseg), row[k + 1]));
+                __stcg(out + i, make_double2(os_row_sum(s_part[r], r < rg ? nsg : nss), row[k + 1]));
             }
             __syncwarp();
             target += (unsigned)min(G, n - 1 - k);

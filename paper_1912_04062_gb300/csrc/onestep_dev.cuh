@@ -133,27 +133,32 @@ SK_DEV void os_rows_any(int cnt, double* base, size_t stride, int i0, int G, int
     }
 }
 
-// A warp's share of the pass over R own rows (the first rg of them in global
-// memory from row gbase on, the others in shared memory): OCW / nseg groups of
-// consecutive rows, nseg segments of the columns each.  Few rows take all
-// warps side by side on the columns; many rows give each warp rows of its own,
-// so that a warp's row sums (5 levels of additions) come once per row and not
-// eight times.
+// A warp's share of the pass over R own rows, the first rg of them in global
+// memory (from row gbase on), the others in shared memory: either kind in
+// OCW / nseg groups of consecutive rows, nseg segments of the columns each.
+// Few rows take all warps side by side on the columns; many rows give each
+// warp rows of its own, so that a warp's row sums (5 levels of additions) come
+// once per row and not eight times.  Global rows keep more segments: the warps
+// then read one row's neighbouring lines together.
 template <int MAXRC>
-SK_DEV void os_pass(int nseg, int R, int rg, double* gbase, double* sbase, int n, int lds, int i0, int G, int k,
+SK_DEV void os_pass(int nsg, int nss, int R, int rg, double* gbase, double* sbase, int n, int lds, int i0, int G, int k,
                     const double2* coef, const double* u, const double* p, const double* x, int warp, int lane,
                     double (*part)[OCW]) {
-    const int groups = OCW / nseg, grp = warp / nseg, seg = warp - grp * nseg;
-    const int lo = R * grp / groups, hi = R * (grp + 1) / groups;
     const int ja = (k + 1) & ~3;
-    const int gl = min(hi, rg);
-    if (lo < gl)
-        os_rows_any<MAXRC, true>(gl - lo, gbase + (size_t)lo * G * n, (size_t)G * n, i0 + lo * G, G, n, k, ja,
-                                 coef + lo, u, p, x, seg, nseg, lane, &part[lo][seg]);
-    const int s0 = max(lo, rg);
-    if (s0 < hi)
-        os_rows_any<MAXRC, false>(hi - s0, sbase + (size_t)(s0 - rg) * lds, lds, i0 + s0 * G, G, n, k, ja, coef + s0,
-                                  u, p, x, seg, nseg, lane, &part[s0][seg]);
+    if (rg > 0) {
+        const int groups = OCW / nsg, grp = warp / nsg, seg = warp - grp * nsg;
+        const int lo = rg * grp / groups, hi = rg * (grp + 1) / groups;
+        if (lo < hi)
+            os_rows_any<MAXRC, true>(hi - lo, gbase + (size_t)lo * G * n, (size_t)G * n, i0 + lo * G, G, n, k, ja,
+                                     coef + lo, u, p, x, seg, nsg, lane, &part[lo][seg]);
+    }
+    if (rg < R) {
+        const int groups = OCW / nss, grp = warp / nss, seg = warp - grp * nss;
+        const int lo = rg + (R - rg) * grp / groups, hi = rg + (R - rg) * (grp + 1) / groups;
+        if (lo < hi)
+            os_rows_any<MAXRC, false>(hi - lo, sbase + (size_t)(lo - rg) * lds, lds, i0 + lo * G, G, n, k, ja,
+                                      coef + lo, u, p, x, seg, nss, lane, &part[lo][seg]);
+    }
 }
 
 // The row sum of the segments, in order.

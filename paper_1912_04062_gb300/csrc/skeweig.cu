@@ -106,7 +106,7 @@ struct Plan {
 };
 
 // Orders that take the direct reduction (measured limits: see make_plan).
-constexpr int ONESTEP_FP64 = 8192, ONESTEP_FP64_VALUES = 5500, ONESTEP_REFINE = 4200, ONESTEP_PARTIAL = 5000,
+constexpr int ONESTEP_FP64 = 8192, ONESTEP_FP64_VALUES = 5500, ONESTEP_REFINE = 6600, ONESTEP_PARTIAL = 5000,
               ONESTEP_VALUES = 3800;
 
 // One carve-up routine serves both sizing (base == nullptr) and placement.
@@ -283,10 +283,17 @@ int run_solve(cudaStream_t st, int n, const double* A, int lda, int nev, double*
             KtScope kt(st, KT_OTHER);
             zero_int_kernel<<<1, 32, 0, st>>>(p.status);
             count_launch();
-            if (const cudaError_t e = onestep_full(st, n, A, lda, p.W, check, p.status)) return cuda_fail(e);
+            if (p.refine) {
+                const int rc = onestep_df_full(st, n, A, lda, p.W, check, p.ws_one, p.sz_one, p.status);
+                if (rc) return rc;
+            } else if (const cudaError_t e = onestep_full(st, n, A, lda, p.W, check, p.status)) {
+                return cuda_fail(e);
+            }
         }
         mark(1);
-        int rc = onestep_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap);
+        // double-float where the refinement follows, FP64 otherwise
+        int rc = p.refine ? onestep_df_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap)
+                          : onestep_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap);
         if (rc) return rc;
         mark(2);
         mark(3);

@@ -59,17 +59,25 @@ def test_direct_route_matches_two_step(n, nev):
     assert torch.equal(lam3, lam1) and torch.equal(Zr3, Zr) and torch.equal(Zi3, Zi)
 
 
-@pytest.mark.parametrize("n", [64, 307, 1002])
-def test_direct_route_refined_is_orthogonal(n):
-    # one refinement iteration follows the direct reduction: it has to leave
-    # the orthogonality of a converged refinement, not the square of the
-    # starting vectors' norm error
+@pytest.mark.parametrize("n,scale,tiny", [(2, 1.0, 1.0), (4, 1.0, 1.0), (64, 1.0, 1.0), (130, 1e-120, 1.0),
+                                          (306, 1e100, 1.0), (308, 1.0, 1e-5), (308, 1.0, 1e-8), (1002, 1.0, 1.0),
+                                          (2070, 1.0, 1.0)])
+def test_direct_route_refined_is_orthogonal(n, scale, tiny):
+    # the double-float reduction and one refinement iteration have to leave
+    # the orthogonality of a converged refinement (not the square of the
+    # starting vectors' norm error), for any scaling of the matrix and with a
+    # block far below its largest entries
     import torch
     import paper_1912_04062_gb300 as sk
-    A = inputs.random_skew(n, seed=7100 + n)
-    dA = sk.fortran(torch.from_numpy(A).cuda())
+    A = inputs.random_skew(n, seed=7100 + n) * scale
+    if tiny != 1.0:
+        h = n // 2
+        A[h:, :h] = 0.0
+        A[:h, h:] = 0.0
+        A[h:, h:] *= tiny
+    dA = sk.fortran(torch.from_numpy(np.asfortranarray(A)).cuda())
     lam, Zr, Zi = _solve(dA, n // 2, sk.Options(mode=sk.SKEW_MODE_MIXED_REFINED))
-    r, o, f = sk.metrics(dA, lam, Zr, Zi)
+    r, o, f = sk.metrics(dA / scale, lam / scale, Zr, Zi)
     assert r <= 50 * n * EPS * f and o <= 5 * n * EPS
 
 
