@@ -100,11 +100,17 @@ def _sha16(rel):
         return None
 
 
-def kind_flops(kind, form, n, nev, b=64):
+def kind_flops(kind, form, n, nev, b=64, direct=False):
     """Algorithmic flops of one solve for the kinds whose launches do not
     carry them (nominal counts: Q_trd 4 n^2 nev, the FP64 form's
     GEMM-type work 4/3 n^3 + 4 n^2 nev, the chase about 6 b n^2, the panel
-    QRs about b n^2); None where no count is defined."""
+    QRs about b n^2); None where no count is defined.  direct: the solve
+    reduced straight to tridiagonal form, so its reduction kernel (kind
+    panel_qr) does 4/3 n^3 and its GEMM-type kernels the back-transformation."""
+    if direct and kind == "panel_qr":
+        return 4.0 / 3.0 * n ** 3
+    if direct and kind == "gemm_f64":
+        return 4.0 * n * n * nev
     if kind == "qtrd":
         return 4.0 * n * n * nev
     if kind == "gemm_f64":
@@ -127,6 +133,8 @@ def select_roofline(kinds, form, n, nev, solves, peaks=None, traffic=None):
     the derived FP32 or FP64 ALU peak for SIMT kernels."""
     peaks = peaks or PEAKS
     per_ms = {k: v[0] / solves for k, v in kinds.items()}
+    # no Q_trd launched: the FP64 form took the direct route
+    direct = form == "fp64" and kinds.get("qtrd", (0, 0, 0))[2] == 0 and kinds.get("panel_qr", (0, 0, 0))[2] > 0
     order = sorted(per_ms, key=per_ms.get, reverse=True)
     for k in order:
         if k not in KIND_KERNELS or per_ms[k] <= 0:
@@ -135,12 +143,14 @@ def select_roofline(kinds, form, n, nev, solves, peaks=None, traffic=None):
         if k == "qtrd":
             arith = "fp32" if form == "mixed" else "fp64"
             name = "qtrd_slide_kernel (FP32)" if form == "mixed" else "qtrd_smem_kernel<double> (FP64)"
+        if k == "panel_qr" and direct:
+            name = "onestep_sym_kernel (FP64 direct reduction)"
         if arith == "tensor":
             fl = kinds[k][1] / solves
             peak, bound = peaks["bf16_tflops_sustained"], "tensor"
             note = f"{peaks.get('source', 'of measured')}: cuBLAS bf16 sustained (kernel timed inside a long step)"
         else:
-            fl = kind_flops(k, form, n, nev)
+            fl = kind_flops(k, form, n, nev, direct=direct)
             if fl is None:
                 continue
             peak = FP32_PEAK_TFLOPS if arith == "fp32" else FP64_PEAK_TFLOPS
@@ -167,12 +177,12 @@ def batched_roofline(sizes, nevs, seconds):
     flops per matrix (tridiagonalisation 4/3 n^3, back-transformation of the
     2 nev real columns through the reflectors 4 n^2 nev; bisection and inverse
     iteration not counted) over the launch time, against the derived FP64 ALU
-    peak (the kernel is FP64 SIMT, one CTA per matrix)."""
+    peak (FP64 SIMT kernels; the stages' launches together)."""
     flops = float(sum(4.0 / 3.0 * n ** 3 + 4.0 * n * n * k for n, k in zip(sizes, nevs)))
     achieved = flops / seconds / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None, "flops": flops,
-            "kernel": "bt_persistent_kernel (FP64 SIMT, one CTA per matrix)",
+            "kernel": "cluster_reduce_kernel and bt_wy_kernel (FP64 SIMT) with the stages between them",
             "peak_note": f"derived FP64 ALU peak: 2 FMA/clk/SM x {SM_COUNT} SMs x {SM_MHZ:.0f} MHz"}
 
 

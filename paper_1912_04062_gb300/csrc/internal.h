@@ -81,6 +81,17 @@ int onestep_df_full(cudaStream_t st, int n, const double* A, int lda, void* F, i
                     int* status);
 int onestep_df_reduce(cudaStream_t st, int n, void* F, double* V, double* tau, double* alpha, void* ws,
                       size_t ws_bytes, int* d_status, unsigned spin_cap);
+// max |A| of the strict lower triangle into *amax (bits of a double, zeroed by
+// the caller; values that are not finite are left out); V from pairs of floats
+// to doubles, in place.
+int onestep_amax(cudaStream_t st, int n, const double* A, int lda, unsigned long long* amax);
+int onestep_widen(cudaStream_t st, size_t count, double* V);
+// The same with the lower triangle only, in memory (onestep_sym.cu): FP64, or
+// double-float (pairs).  Reads A itself.
+int onestep_sym_max();
+size_t onestep_sym_ws(int n);
+int onestep_sym_reduce(cudaStream_t st, int n, const double* A, int lda, bool pairs, double* V, double* tau,
+                       double* alpha, void* ws, size_t ws_bytes, int check, int* d_status, unsigned spin_cap);
 // FP64 Z = H_0 H_1 ... H_{n-3} D Q from the interleaved tridiagonal vectors Qi
 // (Qi[i * nev + k]), for the sizes of onestep_wy_fits.
 bool onestep_wy_fits(int n, int nev);

@@ -99,29 +99,41 @@ struct Plan {
     size_t sz_reduce, sz_chase, sz_tri, sz_qband, sz_refine, sz_qtc;
     bool refine;  // mixed form with a complete basis (n even, nev = n/2)
     bool onestep;  // direct tridiagonalisation instead of band + chase (onestep.cu)
+    bool sym;      // its form for matrices in memory (onestep_sym.cu)
     bool wy;       // its FP64 back-transformation in one launch (else panel products)
     double *V1, *tau1;  // its reflectors
     void *ws_one, *ws_back;
     size_t sz_one, sz_back;
 };
 
-// Orders that take the direct reduction (measured limits: see make_plan).
-constexpr int ONESTEP_FP64 = 8192, ONESTEP_FP64_VALUES = 5500, ONESTEP_REFINE = 6600, ONESTEP_PARTIAL = 5000,
-              ONESTEP_VALUES = 3800;
+// Orders that take the direct reduction.  FP64 with vectors: everywhere it is
+// built for, since the two-step route's Q_trd alone costs as much as its whole
+// back-transformation (n = 8192: 2.01 s against 3.56 s, 4000: 0.28 against 0.71).
+// FP64 values only: the reduction against band reduction and chase (8192: 974
+// against 977 ms, 4000: 134 against 228).  Refined: 8192 0.50 s against 0.75 s,
+// 12288 1.78 against 1.82, 16384 3.98 against 3.61; partial vectors take the FP64
+// form against products of 8 slices (5000: equal; 6001: 400 against 332 ms with
+// the chase and Q_trd), as do values only (4000: 146 against 147 ms).
+constexpr int ONESTEP_FP64 = 16384, ONESTEP_FP64_VALUES = 8000, ONESTEP_REFINE = 11500, ONESTEP_PARTIAL = 5000,
+              ONESTEP_VALUES = 4100;
+// Orders above which the direct reduction keeps the lower triangle only: FP64
+// 3002 67 against 67 ms, 4096 139 against 152; pairs 3002 37.6 against 35.0,
+// 4096 63 against 84.
+constexpr int SYM_FP64 = 3000, SYM_REFINE = 3200;
 
 // One carve-up routine serves both sizing (base == nullptr) and placement.
 bool carve_plan(Plan& p, Carve& cv) {
     const size_t n = (size_t)p.n, b = (size_t)p.b;
     const size_t nn = n ? n : 1;
     p.status = cv.take<int>(16);
-    p.W = cv.take<double>(nn * nn);
+    p.W = p.sym ? nullptr : cv.take<double>(nn * nn);
     if (p.onestep) {
         const size_t vc = (size_t)onestep_vcols(p.n), ne = (size_t)(p.nev ? p.nev : 1);
         p.V1 = cv.take<double>(vc * nn);
         p.tau1 = cv.take<double>(vc);
         p.alpha = cv.take<double>(nn);
         p.Qi = p.vectors ? cv.take<double>(nn * ne) : nullptr;
-        p.sz_one = onestep_ws(p.n);
+        p.sz_one = p.sym ? onestep_sym_ws(p.n) : onestep_ws(p.n);
         p.ws_one = cv.take<char>(p.sz_one);
         p.sz_tri = tridiag_ws(p.n, p.nev);
         p.ws_tri = cv.take<char>(p.sz_tri);
@@ -222,7 +234,8 @@ Plan make_plan(int n, int nev, const skew_opts* o, bool vectors) {
     // unless it names the mode's own choice
     const bool any_qtrd = !o || o->qtrd == SKEW_QTRD_AUTO ||
                           (refined_mode && vectors && !p.refine && o->qtrd == SKEW_QTRD_DF);
-    p.onestep = p.b == 64 && (!p.mixed || refined_mode) && any_qtrd && n >= 2 && n <= lim && n <= onestep_max();
+    p.onestep = p.b == 64 && (!p.mixed || refined_mode) && any_qtrd && n >= 2 && n <= lim && n <= onestep_sym_max();
+    p.sym = p.onestep && n > (p.refine ? SYM_REFINE : SYM_FP64);
     p.wy = p.onestep && vectors && !p.mixed && onestep_wy_fits(n, nev);
     return p;
 }
@@ -283,7 +296,8 @@ int run_solve(cudaStream_t st, int n, const double* A, int lda, int nev, double*
             KtScope kt(st, KT_OTHER);
             zero_int_kernel<<<1, 32, 0, st>>>(p.status);
             count_launch();
-            if (p.refine) {
+            if (p.sym) {
+            } else if (p.refine) {
                 const int rc = onestep_df_full(st, n, A, lda, p.W, check, p.ws_one, p.sz_one, p.status);
                 if (rc) return rc;
             } else if (const cudaError_t e = onestep_full(st, n, A, lda, p.W, check, p.status)) {
@@ -292,8 +306,11 @@ int run_solve(cudaStream_t st, int n, const double* A, int lda, int nev, double*
         }
         mark(1);
         // double-float where the refinement follows, FP64 otherwise
-        int rc = p.refine ? onestep_df_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap)
-                          : onestep_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap);
+        int rc = p.sym ? onestep_sym_reduce(st, n, A, lda, p.refine, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, check,
+                                            p.status, spin_cap)
+               : p.refine
+                     ? onestep_df_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap)
+                     : onestep_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap);
         if (rc) return rc;
         mark(2);
         mark(3);
