@@ -222,149 +222,170 @@ __host__ __device__ inline int cl_rows(int n, int G) {
     return fit < rmax ? fit : rmax;
 }
 
-__global__ void __launch_bounds__(CT, 1)
-cluster_reduce_kernel(const BItem* __restrict__ items, const int* __restrict__ order, int count,
-                      int* __restrict__ next) {
+// One matrix by the cluster.  S: its rows that do not fit in shared memory.
+// check: values that are not finite are reported in *status.
+SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, double* S, double* V, double* tau,
+                                double* alpha, int check, int* status) {
     extern __shared__ __align__(16) double cl_sm[];
     __shared__ double s_part[CMAXR][OCW];
     __shared__ double2 s_coef[CMAXR];  // sigma u_i, -sigma p_i of the own rows
     __shared__ double s_red[4];
     __shared__ double s_sc[4];
-    __shared__ int s_q;
     const int G = (int)cl_size(), g = (int)cl_rank();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int ldn = cl_ld(n);
+    double* u = cl_sm;
+    double* p = u + ldn;
+    double* x = p + ldn;
+    double2* qa = reinterpret_cast<double2*>(x + ldn);  // 2 n, double-buffered
+    double* rows = x + 5 * ldn;
+    const int srows = cl_rows(n, G);
+    const int Rt = g < n ? (n - 1 - g) / G + 1 : 0;  // own rows: none past a small order
+    const int rs0 = Rt > srows ? Rt - srows : 0, ilast = g + (Rt - 1) * G;
+    // own rows of the full skew matrix: -A(j, i) right of the diagonal
+    // (contiguous), A(i, j) left of it
+    for (int r = 0; r < Rt; r++) {
+        const int i = g + r * G;
+        double* row = r >= rs0 ? rows + (size_t)(r - rs0) * ldn : S + (size_t)i * n;
+        for (int j = t; j < n; j += CT) {
+            const double v = j > i ? -A[(size_t)i * lda + j] : j < i ? A[(size_t)j * lda + i] : 0.0;
+            if (check && !isfinite(v)) sk_set_error(status, SKEW_ERR_NONFINITE);
+            row[j] = v;
+        }
+    }
+    // zeros of V above the reflectors and in the columns that fill up the
+    // last panel (the values come after the first barrier below)
+    const int vc = bt_vcols(n);
+    for (int c = g; c < vc; c += G) {
+        const int hi = c < n - 2 ? c + 1 : n;
+        for (int i = t; i < hi; i += CT) V[(size_t)c * n + i] = 0.0;
+    }
+    if (g == 0)
+        for (int c = n - 2 + t; c < vc; c += CT) tau[c] = 0.0;
+    double beta = 0.0, sigma = 0.0;
+    for (int k = 0; k + 1 < n; k++) {
+        const bool act = ilast > k;  // rows left
+        const int rf = (k + 1 > g) ? (k + 1 - g + G - 1) / G : 0, R = Rt - rf;
+        if (act) {
+            const double2* in = qa + (size_t)(k & 1) * n;
+            if (k == 0) {
+                for (int j = t; j < n; j += CT) {
+                    x[j] = j > 0 ? A[j] : 0.0;
+                    u[j] = 0.0;
+                    p[j] = 0.0;
+                }
+            } else {
+                const double2 qk = in[k];
+                const double uk = -sigma * u[k], pk = sigma * fma(-beta, qk.y, qk.x);
+                for (int j = k + 1 + t; j < n; j += CT) {
+                    const double2 e = in[j];
+                    const double pj = fma(-beta, e.y, e.x);
+                    p[j] = pj;
+                    x[j] = fma(u[j], pk, fma(pj, uk, e.y));
+                }
+            }
+        }
+        __syncthreads();
+        if (k == n - 2) {
+            if (act && t == 0) alpha[k] = -x[n - 1];
+            break;
+        }
+        const int rg = max(rs0, rf) - rf;  // rows of global memory
+        // a function of the order left alone: a matrix's result does not
+        // depend on the size of the cluster
+        const int m = n - k - 1, nseg = m >= 288 ? 1 : m >= 144 ? 2 : m >= 72 ? 4 : 8;
+        if (act && warp < OCW) {
+            for (int r = t; r < R; r += 256)
+                s_coef[r] = make_double2(sigma * u[g + (rf + r) * G], -sigma * p[g + (rf + r) * G]);
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            os_pass<4>(nseg, nseg, R, rg, S + (size_t)(g + rf * G) * n, rows + (size_t)(rf + rg - rs0) * ldn, n, ldn,
+                       g + rf * G, G, k, s_coef, u, p, x, warp, lane, s_part);
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            // publish (q_i, a_i) of the own rows to every CTA
+            double2* out = qa + (size_t)((k + 1) & 1) * n;
+            for (int r = t; r < R; r += 256) {
+                const int i = g + (rf + r) * G;
+                const double* row = r >= rg ? rows + (size_t)(rf + r - rs0) * ldn : S + (size_t)i * n;
+                const double sum = os_row_sum(s_part[r], nseg);
+                const double av = row[k + 1];
+                for (int c = 0; c < G; c++)
+                    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(cl_map(out + i, (uint32_t)c)),
+                                 "d"(sum), "d"(av)
+                                 : "memory");
+            }
+        } else if (act) {
+            // the norm of x below its first element, beta and sigma
+            double nr = 0.0;
+            for (int j = k + 2 + (t - 256); j < n; j += 128) nr = fma(x[j], x[j], nr);
+            nr = sk_warp_sum(nr);
+            if (lane == 0) s_red[warp - OCW] = nr;
+            asm volatile("bar.sync 2, 128;" ::: "memory");
+            if (t == 256) {
+                const double s2 = (s_red[0] + s_red[1]) + (s_red[2] + s_red[3]);
+                const double x0 = x[k + 1];
+                double b = x0, sg = 0.0, inv = 0.0;
+                if (s2 != 0.0) {
+                    const double rr = sqrt(fma(x0, x0, s2));
+                    b = (x0 >= 0.0) ? -rr : rr;
+                    // this chain is the longest of a column at small orders
+                    const double den = b * (x0 - b);
+                    sg = den > -1e270 && den < -1e-270 ? -tri::rcp_fast(den) : -1.0 / den;
+                    inv = -sg * b;
+                }
+                s_sc[0] = b;
+                s_sc[1] = sg;
+                s_sc[2] = inv;
+                s_sc[3] = x0 - b;
+            }
+        }
+        cl_barrier();
+        if (act) {
+            beta = s_sc[0];
+            sigma = s_sc[1];
+            const double inv = s_sc[2], u0 = s_sc[3];
+            for (int r = t; r < R; r += CT) {
+                const int i = g + (rf + r) * G;
+                V[(size_t)k * n + i] = (i == k + 1) ? 1.0 : x[i] * inv;
+            }
+            if (ilast == n - 1 && t == 0) {
+                tau[k] = sigma * u0 * u0;
+                alpha[k] = -beta;
+            }
+            if (t == 0) x[k + 1] = u0;  // x_0 itself is not read above
+            double* sw = u;
+            u = x;
+            x = sw;
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(CT, 1)
+cluster_reduce_kernel(const BItem* __restrict__ items, const int* __restrict__ order, int count,
+                      int* __restrict__ next) {
+    __shared__ int s_q;
     for (;;) {
         cl_barrier();  // nobody writes into this CTA's shared memory any more
-        if (g == 0 && t == 0) {
+        if (cl_rank() == 0 && threadIdx.x == 0) {
             const int q = atomicAdd(next, 1);
-            for (int c = 0; c < G; c++)
-                asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cl_map(&s_q, (uint32_t)c)), "r"(q) : "memory");
+            for (uint32_t c = 0; c < cl_size(); c++)
+                asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cl_map(&s_q, c)), "r"(q) : "memory");
         }
         cl_barrier();
         const int q = s_q;
         if (q >= count) return;
         const BItem it = items[order[q]];
-        const int n = it.n, ldn = cl_ld(n);
-        double* u = cl_sm;
-        double* p = u + ldn;
-        double* x = p + ldn;
-        double2* qa = reinterpret_cast<double2*>(x + ldn);  // 2 n, double-buffered
-        double* rows = x + 5 * ldn;
-        const int srows = cl_rows(n, G);
-        const int Rt = (n - 1 - g) / G + 1, rs0 = Rt > srows ? Rt - srows : 0;
-        const int ilast = g + (Rt - 1) * G;
-        // own rows of the full skew matrix: -A(j, i) right of the diagonal
-        // (contiguous), A(i, j) left of it
-        for (int r = 0; r < Rt; r++) {
-            const int i = g + r * G;
-            double* row = r >= rs0 ? rows + (size_t)(r - rs0) * ldn : it.S + (size_t)i * n;
-            for (int j = t; j < n; j += CT)
-                row[j] = j > i ? -it.A[(size_t)i * it.lda + j] : j < i ? it.A[(size_t)j * it.lda + i] : 0.0;
-        }
-        // zeros of V above the reflectors and in the columns that fill up the
-        // last panel (the values come after the first barrier below)
-        const int vc = bt_vcols(n);
-        for (int c = g; c < vc; c += G) {
-            const int hi = c < n - 2 ? c + 1 : n;
-            for (int i = t; i < hi; i += CT) it.V[(size_t)c * n + i] = 0.0;
-        }
-        if (g == 0)
-            for (int c = n - 2 + t; c < vc; c += CT) it.tau[c] = 0.0;
-        double beta = 0.0, sigma = 0.0;
-        for (int k = 0; k + 1 < n; k++) {
-            const bool act = ilast > k;  // rows left
-            const int rf = (k + 1 > g) ? (k + 1 - g + G - 1) / G : 0, R = Rt - rf;
-            if (act) {
-                const double2* in = qa + (size_t)(k & 1) * n;
-                if (k == 0) {
-                    for (int j = t; j < n; j += CT) {
-                        x[j] = j > 0 ? it.A[j] : 0.0;
-                        u[j] = 0.0;
-                        p[j] = 0.0;
-                    }
-                } else {
-                    const double2 qk = in[k];
-                    const double uk = -sigma * u[k], pk = sigma * fma(-beta, qk.y, qk.x);
-                    for (int j = k + 1 + t; j < n; j += CT) {
-                        const double2 e = in[j];
-                        const double pj = fma(-beta, e.y, e.x);
-                        p[j] = pj;
-                        x[j] = fma(u[j], pk, fma(pj, uk, e.y));
-                    }
-                }
-            }
-            __syncthreads();
-            if (k == n - 2) {
-                if (act && t == 0) it.alpha[k] = -x[n - 1];
-                break;
-            }
-            const int rg = max(rs0, rf) - rf;  // rows of global memory
-            // a function of the order left alone: a matrix's result does not
-            // depend on the size of the cluster
-            const int m = n - k - 1, nseg = m >= 288 ? 1 : m >= 144 ? 2 : m >= 72 ? 4 : 8;
-            if (act && warp < OCW) {
-                for (int r = t; r < R; r += 256)
-                    s_coef[r] = make_double2(sigma * u[g + (rf + r) * G], -sigma * p[g + (rf + r) * G]);
-                asm volatile("bar.sync 1, 256;" ::: "memory");
-                os_pass<4>(nseg, nseg, R, rg, it.S + (size_t)(g + rf * G) * n, rows + (size_t)(rf + rg - rs0) * ldn, n, ldn,
-                           g + rf * G, G, k, s_coef, u, p, x, warp, lane, s_part);
-                asm volatile("bar.sync 1, 256;" ::: "memory");
-                // publish (q_i, a_i) of the own rows to every CTA
-                double2* out = qa + (size_t)((k + 1) & 1) * n;
-                for (int r = t; r < R; r += 256) {
-                    const int i = g + (rf + r) * G;
-                    const double* row = r >= rg ? rows + (size_t)(rf + r - rs0) * ldn : it.S + (size_t)i * n;
-                    const double sum = os_row_sum(s_part[r], nseg);
-                    const double av = row[k + 1];
-                    for (int c = 0; c < G; c++)
-                        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(cl_map(out + i, (uint32_t)c)),
-                                     "d"(sum), "d"(av)
-                                     : "memory");
-                }
-            } else if (act) {
-                // the norm of x below its first element, beta and sigma
-                double nr = 0.0;
-                for (int j = k + 2 + (t - 256); j < n; j += 128) nr = fma(x[j], x[j], nr);
-                nr = sk_warp_sum(nr);
-                if (lane == 0) s_red[warp - OCW] = nr;
-                asm volatile("bar.sync 2, 128;" ::: "memory");
-                if (t == 256) {
-                    const double s2 = (s_red[0] + s_red[1]) + (s_red[2] + s_red[3]);
-                    const double x0 = x[k + 1];
-                    double b = x0, sg = 0.0, inv = 0.0;
-                    if (s2 != 0.0) {
-                        const double rr = sqrt(fma(x0, x0, s2));
-                        b = (x0 >= 0.0) ? -rr : rr;
-                        sg = -1.0 / (b * (x0 - b));
-                        inv = -sg * b;
-                    }
-                    s_sc[0] = b;
-                    s_sc[1] = sg;
-                    s_sc[2] = inv;
-                    s_sc[3] = x0 - b;
-                }
-            }
-            cl_barrier();
-            if (act) {
-                beta = s_sc[0];
-                sigma = s_sc[1];
-                const double inv = s_sc[2], u0 = s_sc[3];
-                for (int r = t; r < R; r += CT) {
-                    const int i = g + (rf + r) * G;
-                    it.V[(size_t)k * n + i] = (i == k + 1) ? 1.0 : x[i] * inv;
-                }
-                if (ilast == n - 1 && t == 0) {
-                    it.tau[k] = sigma * u0 * u0;
-                    it.alpha[k] = -beta;
-                }
-                if (t == 0) x[k + 1] = u0;  // x_0 itself is not read above
-                double* sw = u;
-                u = x;
-                x = sw;
-            }
-            __syncthreads();
-        }
+        cluster_reduce_body(it.n, it.A, it.lda, it.S, it.V, it.tau, it.alpha, 0, nullptr);
     }
+}
+
+// One matrix, one cluster.
+__global__ void __launch_bounds__(CT, 1)
+cluster_reduce_one_kernel(int n, const double* __restrict__ A, int lda, double* V, double* tau, double* alpha,
+                          int check, int* status) {
+    cl_barrier();  // every CTA of the cluster has started
+    cluster_reduce_body(n, A, lda, nullptr, V, tau, alpha, check, status);
+    cl_barrier();  // no CTA leaves while another may still write to it
 }
 
 // ---- eigenvalues and vectors of every tridiagonal ----------------------------
@@ -710,11 +731,42 @@ int pick_clusters(const std::vector<int>& ns, BatchPlanDev* out) {
 
 }  // namespace
 
+int cluster_reduce(cudaStream_t st, int n, const double* A, int lda, double* V, double* tau, double* alpha, int check,
+                   int* d_status) {
+    if (n < 2 || n > CLUSTER_ONE_MAX) return SKEW_ERR_UNSUPPORTED;
+    auto kern = cluster_reduce_one_kernel;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CSMEM) != cudaSuccess)
+        return SKEW_ERR_LAUNCH;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+    KtScope kt(st, KT_PANEL_QR);
+    for (int G = 16; G >= 8; G /= 2) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)G);
+        cfg.blockDim = dim3(CT);
+        cfg.dynamicSmemBytes = CSMEM;
+        cfg.stream = st;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)G;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, n, A, lda, V, tau, alpha, check, d_status);
+        if (e == cudaSuccess) {
+            count_launch();
+            return 0;
+        }
+        cudaGetLastError();
+        if (G == 8) return cuda_fail(e);
+    }
+    return SKEW_ERR_LAUNCH;
+}
+
 // Launch parameters for a configuration (sets the kernels' attributes; no
 // stream work).
 int batched_prepare(const BatchPlanDev& d, const skew_batched_config& cfg, BatchLaunch* out) {
     if (batched_config_check(cfg)) return SKEW_ERR_UNSUPPORTED;
-    const int dyn_wy = (int)wy_smem(d.nmax, BE);
+    const int dyn_wy = (int)wy_smem(BATCH_MAX, BE);  // a constant: plans of several threads share the kernel
     if (cudaFuncSetAttribute(bt_wy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_wy) != cudaSuccess)
         return SKEW_ERR_LAUNCH;
     // the shared-memory threshold cannot exceed what the per-SM budget allows

@@ -78,26 +78,6 @@ SK_DEV bool sk_grid_barrier(unsigned* counter, unsigned& epoch, int* status, uns
     return s_ok != 0;
 }
 
-// Wait until *flag >= want (acquire).  Thread 0 polls; the block synchronises.
-SK_DEV bool sk_wait_flag_geq(const int* flag, int want, int* status) {
-    __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        unsigned polls = 0;
-        while (sk_ld_acquire_s32(flag) < want) {
-            if (++polls > SK_SPIN_CAP || *(volatile int*)status != 0) {
-                ok = 0;
-                break;
-            }
-            __nanosleep(32);
-        }
-        if (!ok) sk_set_error(status, SKEW_ERR_DEVICE_TIMEOUT);
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
 template <typename T>
 SK_DEV T sk_warp_sum(T v) {
 #pragma unroll

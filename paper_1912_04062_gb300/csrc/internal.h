@@ -61,8 +61,6 @@ int num_panels(int n, int b);
 cudaError_t tfactor_panels(cudaStream_t st, int panels, const double* tau, const double* G, double* T);
 
 // ---- onestep.cu (direct tridiagonalisation, FP64) ---------------------------
-// Largest order it takes.
-int onestep_max();
 size_t onestep_ws(int n);
 // Columns of V (and entries of tau): n - 2 rounded up to whole panels of 64.
 int onestep_vcols(int n);
@@ -76,7 +74,6 @@ int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, do
 // The same in double-float (onestep_df.cu) for a caller that refines the
 // result: F holds pairs of floats (8 bytes an element); ws is shared by the two
 // calls (onestep_ws bytes) and carries the scaling from one to the other.
-int onestep_df_max();
 int onestep_df_full(cudaStream_t st, int n, const double* A, int lda, void* F, int check, void* ws, size_t ws_bytes,
                     int* status);
 int onestep_df_reduce(cudaStream_t st, int n, void* F, double* V, double* tau, double* alpha, void* ws,
@@ -289,6 +286,14 @@ cudaError_t bse_jl(cudaStream_t st, int h, double* L, int ld, double* JL, int ld
 cudaError_t trsm_lower_t(cudaStream_t st, int N, const double* L, int ld, double* X, int ldx, int ncols);
 cudaError_t bse_psi(cudaStream_t st, int h, int nev, const double* Xr, const double* Xi, int ldx,
                     const double* lambda, double* Pr, double* Pi, int ldp);
+
+// Reduction of one small matrix by one cluster (batched.cu's kernel; outputs as
+// onestep_reduce).  Its exchange takes 300 clocks instead of 3000, but 16 SMs do
+// the work of 152: 2.9 us a column against 3.8 at n = 48, 3.6 against 3.9 at 200,
+// 4.5 against 4.0 at 300.
+constexpr int CLUSTER_ONE_MAX = 220;
+int cluster_reduce(cudaStream_t st, int n, const double* A, int lda, double* V, double* tau, double* alpha, int check,
+                   int* d_status);
 
 // ---- metrics.cu -------------------------------------------------------------
 size_t metrics_ws(int n, int nev, int s);

@@ -39,6 +39,10 @@ namespace {
 
 constexpr int OT = 256;     // threads of the reduction kernel
 constexpr int OMAXR = 64;   // rows of one CTA at most (n <= 64 G)
+// Dynamic shared memory at most: of 227 KB, the static arrays take about 5.3 KB.
+// The kernels' limits are set to constants, so that calls of several threads
+// cannot take them from one another.
+constexpr int OS_SMEM = 221 * 1024, WY_SMEM = 226 * 1024;
 
 struct OsArgs {
     int n;
@@ -86,10 +90,25 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
                 p[j] = 0.0;
             }
         } else {
+            // two elements are under way while element k is waited for
+            const int j0 = k + 1 + t, j1 = j0 + OT;
+            double2 e0 = make_double2(0.0, 0.0), e1 = e0;
+            if (j0 < n) e0 = __ldcg(qa + j0);
+            if (j1 < n) e1 = __ldcg(qa + j1);
             const double2 qk = __ldcg(qa + k);
             const double uk = -sigma * u[k], pk = sigma * fma(-beta, qk.y, qk.x);
+            if (j0 < n) {
+                const double pj = fma(-beta, e0.y, e0.x);
+                p[j0] = pj;
+                x[j0] = fma(u[j0], pk, fma(pj, uk, e0.y));
+            }
+            if (j1 < n) {
+                const double pj = fma(-beta, e1.y, e1.x);
+                p[j1] = pj;
+                x[j1] = fma(u[j1], pk, fma(pj, uk, e1.y));
+            }
 #pragma unroll 4
-            for (int j = k + 1 + t; j < n; j += OT) {
+            for (int j = j1 + OT; j < n; j += OT) {
                 const double2 e = __ldcg(qa + j);
                 const double pj = fma(-beta, e.y, e.x);
                 p[j] = pj;
@@ -248,7 +267,7 @@ template <int E>
 cudaError_t wy_launch(cudaStream_t st, int n, int nev, const double* V, const double* Gt, const double* tau,
                       const double* Qi, double* Zre, double* Zim, int ldz) {
     const size_t dyn = wy_smem(n, E);
-    if (const cudaError_t e = cudaFuncSetAttribute(os_wy_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn))
+    if (const cudaError_t e = cudaFuncSetAttribute(os_wy_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, WY_SMEM))
         return e;
     os_wy_kernel<E><<<(nev + E - 1) / E, WT, dyn, st>>>(n, nev, V, Gt, tau, Qi, Zre, Zim, ldz);
     count_launch();
@@ -258,14 +277,12 @@ cudaError_t wy_launch(cudaStream_t st, int n, int nev, const double* V, const do
 int os_srows(int n, int G) {
     const int rmax = (n + G - 1) / G;
     const size_t vec = 3 * sizeof(double) * (size_t)(n | 1), row = sizeof(double) * (size_t)(n | 1);
-    const size_t cap = 221 * 1024;  // of 227 KB: the static arrays take about 5.3 KB
+    const size_t cap = OS_SMEM;
     const int fit = vec + row > cap ? 0 : (int)((cap - vec) / row);
     return std::min(rmax, fit);
 }
 
 }  // namespace
-
-int onestep_max() { return std::min(OMAXR * device_sms(), 9000); }
 
 size_t onestep_ws(int n) {
     Carve cv(nullptr, ~size_t(0));
@@ -308,7 +325,7 @@ int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, do
     o.srows = os_srows(n, G);
     const size_t dyn = sizeof(double) * (size_t)(n | 1) * (3 + (size_t)o.srows);
     if (const cudaError_t e =
-            cudaFuncSetAttribute(onestep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn))
+            cudaFuncSetAttribute(onestep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OS_SMEM))
         return cuda_fail(e);
     void* args[] = {&o};
     KtScope kt(st, KT_PANEL_QR);
@@ -322,7 +339,7 @@ int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, do
 static int wy_e(int n, int nev) {
     const int sms = device_sms();
     const int e = (nev + sms - 1) / sms;
-    return (e <= 6 && wy_smem(n, e) <= 226 * 1024) ? e : 0;
+    return (e <= 6 && wy_smem(n, e) <= (size_t)WY_SMEM) ? e : 0;
 }
 
 bool onestep_wy_fits(int n, int nev) { return wy_e(n, nev) > 0; }

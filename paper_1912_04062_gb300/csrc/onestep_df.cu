@@ -28,6 +28,7 @@ namespace {
 
 constexpr int DT = 512, DW = DT / 32;  // sixteen warps: the pass waits for L2, not for the FP32 pipe
 constexpr int DMAXR = 64;
+constexpr int DF_SMEM = 216 * 1024;  // dynamic shared memory at most: the static arrays take about 9.5 KB of 227
 
 struct DfArgs {
     int n;
@@ -384,7 +385,7 @@ df_full_kernel(int n, const double* __restrict__ A, int lda, const unsigned long
 int df_srows(int n, int G) {
     const int rmax = (n + G - 1) / G;
     const size_t vec = 3 * sizeof(float2) * (size_t)(n | 1), row = sizeof(float2) * (size_t)(n | 1);
-    const size_t cap = 216 * 1024;  // of 227 KB: the static arrays take about 9.5 KB
+    const size_t cap = DF_SMEM;
     const int fit = vec + row > cap ? 0 : (int)((cap - vec) / row);
     return std::min(rmax, fit);
 }
@@ -402,8 +403,6 @@ int onestep_widen(cudaStream_t st, size_t count, double* V) {
     count_launch();
     return cuda_ok(cudaGetLastError());
 }
-
-int onestep_df_max() { return std::min(DMAXR * device_sms(), 9000); }
 
 int onestep_df_full(cudaStream_t st, int n, const double* A, int lda, void* F, int check, void* ws, size_t ws_bytes,
                     int* status) {
@@ -445,7 +444,7 @@ int onestep_df_reduce(cudaStream_t st, int n, void* F, double* V, double* tau, d
     o.srows = df_srows(n, G);
     const size_t dyn = sizeof(float2) * (size_t)(n | 1) * (3 + (size_t)o.srows);
     if (const cudaError_t e =
-            cudaFuncSetAttribute(onestep_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn))
+            cudaFuncSetAttribute(onestep_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DF_SMEM))
         return cuda_fail(e);
     void* args[] = {&o};
     KtScope kt(st, KT_PANEL_QR);

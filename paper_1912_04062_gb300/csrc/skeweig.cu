@@ -1,6 +1,6 @@
 // skeweig.cu -- C ABI of the skew-symmetric eigensolver: argument checks,
-// workspace carve-up and the stage sequence of Algorithm 1 (two-step form) on
-// one stream.
+// workspace carve-up and the stage sequence of Algorithm 1 (direct or two-step
+// reduction, by order and mode) on one stream.
 #include <atomic>
 #include <cstdint>
 #include <mutex>
@@ -100,6 +100,7 @@ struct Plan {
     bool refine;  // mixed form with a complete basis (n even, nev = n/2)
     bool onestep;  // direct tridiagonalisation instead of band + chase (onestep.cu)
     bool sym;      // its form for matrices in memory (onestep_sym.cu)
+    bool cluster;  // its form for small orders (one thread-block cluster, FP64)
     bool wy;       // its FP64 back-transformation in one launch (else panel products)
     double *V1, *tau1;  // its reflectors
     void *ws_one, *ws_back;
@@ -126,7 +127,7 @@ bool carve_plan(Plan& p, Carve& cv) {
     const size_t n = (size_t)p.n, b = (size_t)p.b;
     const size_t nn = n ? n : 1;
     p.status = cv.take<int>(16);
-    p.W = p.sym ? nullptr : cv.take<double>(nn * nn);
+    p.W = p.sym || p.cluster ? nullptr : cv.take<double>(nn * nn);
     if (p.onestep) {
         const size_t vc = (size_t)onestep_vcols(p.n), ne = (size_t)(p.nev ? p.nev : 1);
         p.V1 = cv.take<double>(vc * nn);
@@ -236,15 +237,27 @@ Plan make_plan(int n, int nev, const skew_opts* o, bool vectors) {
                           (refined_mode && vectors && !p.refine && o->qtrd == SKEW_QTRD_DF);
     p.onestep = p.b == 64 && (!p.mixed || refined_mode) && any_qtrd && n >= 2 && n <= lim && n <= onestep_sym_max();
     p.sym = p.onestep && n > (p.refine ? SYM_REFINE : SYM_FP64);
+    p.cluster = p.onestep && n <= CLUSTER_ONE_MAX;
     p.wy = p.onestep && vectors && !p.mixed && onestep_wy_fits(n, nev);
     return p;
 }
 
+// Bytes for (n, nev), never less than for a smaller order: the routes differ in
+// what they hold, and a workspace taken for the largest of several orders has
+// to serve the others.
 size_t plan_bytes(int n, int nev, const skew_opts* o, bool vectors) {
-    Plan p = make_plan(n, nev, o, vectors);
-    Carve cv(nullptr, ~size_t(0));
-    carve_plan(p, cv);
-    return cv.off + 256;
+    auto one = [&](int m) {
+        Plan p = make_plan(m, m < n && nev > m / 2 ? m / 2 : nev, o, vectors);
+        Carve cv(nullptr, ~size_t(0));
+        carve_plan(p, cv);
+        return cv.off;
+    };
+    size_t bytes = one(n);
+    // the last orders of each route
+    for (int m : {CLUSTER_ONE_MAX, SYM_FP64, SYM_REFINE, ONESTEP_VALUES, ONESTEP_PARTIAL, ONESTEP_FP64_VALUES,
+                  ONESTEP_REFINE, ONESTEP_FP64})
+        if (m < n) bytes = one(m) > bytes ? one(m) : bytes;
+    return bytes + 256;
 }
 
 __global__ void f64_to_f32_kernel(size_t count, const double* __restrict__ x, float* __restrict__ y) {
@@ -296,7 +309,8 @@ int run_solve(cudaStream_t st, int n, const double* A, int lda, int nev, double*
             KtScope kt(st, KT_OTHER);
             zero_int_kernel<<<1, 32, 0, st>>>(p.status);
             count_launch();
-            if (p.sym) {
+            if (p.sym || p.cluster) {
+                // these forms read A themselves
             } else if (p.refine) {
                 const int rc = onestep_df_full(st, n, A, lda, p.W, check, p.ws_one, p.sz_one, p.status);
                 if (rc) return rc;
@@ -306,7 +320,8 @@ int run_solve(cudaStream_t st, int n, const double* A, int lda, int nev, double*
         }
         mark(1);
         // double-float where the refinement follows, FP64 otherwise
-        int rc = p.sym ? onestep_sym_reduce(st, n, A, lda, p.refine, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, check,
+        int rc = p.cluster ? cluster_reduce(st, n, A, lda, p.V1, p.tau1, p.alpha, check, p.status)
+               : p.sym ? onestep_sym_reduce(st, n, A, lda, p.refine, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, check,
                                             p.status, spin_cap)
                : p.refine
                      ? onestep_df_reduce(st, n, p.W, p.V1, p.tau1, p.alpha, p.ws_one, p.sz_one, p.status, spin_cap)

@@ -4,30 +4,32 @@
 // Algorithm 1 step 3.
 //
 // Sec. 3 (the solver BSEPACK adapted from ScaLAPACK): bisection + inverse
-// iteration.
-//   * Bisection: Sturm counts from the LDL^T pivots d_0 = -x,
-//     d_i = -x - alpha_{i-1}^2/d_{i-1} (tiny pivots replaced by -pivmin) on
-//     [-g, g], g = ||S||_1, for the nev largest eigenvalues.  GB300 runs FP64
-//     at 1/64 of the FP32 rate and the FP64 recurrence is latency-bound
-//     (the division chain), so the counts run in three precisions: FP32
-//     counts of S / g bracket each eigenvalue to 8 eps32 (four lanes
-//     multisect), double-float counts (FP32 pairs) check the bracket widened
-//     by 64 eps32 and narrow it to 2^-42, and, where the eigenvalues are not
-//     refined afterwards, FP64 counts check it again (widened by 2^-36 g) and
-//     finish it with two-lane multisection.  Each floating-point Sturm count
-//     is exact for a matrix perturbed by a few units of its roundoff
-//     (Kahan), hence the widening before each check.
-//   * Inverse iteration: Gaussian elimination with partial pivoting of
-//     S - lambda I (pivots below eps g raised to eps g), a counter-based
-//     (splitmix64) start vector, at most maxit solves, one extra solve after
-//     the growth test passes.  Eigenvalues closer than ctol form a cluster: a
-//     lone eigenvalue's vector is one thread's work; a cluster's members
-//     iterate in lockstep (each member's solves on its own thread, then the
-//     cluster's CTA orthogonalises them in index order by modified
-//     Gram-Schmidt, normalises them and applies the growth test).
-//     The largest-modulus entry of each vector is made positive.  When the
-//     vectors are refined afterwards, the same steps run in double-float
-//     arithmetic (eps = 2^-44).
+// iteration, each in the form that suits a slow FP64 pipe.
+//   * Eigenvalues: Sturm counts for the nev largest on [-g, g], g = ||S||_1.
+//     FP64 runs at 1/64 of the FP32 rate and the recurrence is a division
+//     chain, so FP32 counts of S / g bracket each eigenvalue to 8 eps32 first
+//     (four lanes multisect).  Where the vectors are not refined, FP64 counts
+//     on the zero-diagonal form check the bracket, widened by 64 eps32, and
+//     finish it with 2 to 32 lanes an eigenvalue, as many as fill the FP64
+//     pipes (32 lanes: a factor 33 a count, 7 counts instead of 30); where they
+//     are, double-float counts (FP32 pairs) narrow it to 2^-42.  Each floating-point Sturm count is
+//     exact for a matrix perturbed by a few units of its roundoff (Kahan),
+//     hence the widening before each check.
+//   * Vectors: the twisted factorisation of S - lambda I (stationary and
+//     progressive transforms met at the row of the smallest |gamma|: Fernando;
+//     Parlett and Dhillon), FP64, two lanes a vector, and where no refinement
+//     follows one more solve with it (one shot alone: orthogonality 3.2 n eps
+//     at n = 1001, with the solve 0.3): two passes each way instead of two or
+//     three pivoted LU solves.  Vectors closer than ctol are a cluster: gaps above 1e-9 g
+//     leave them independent and one modified Gram-Schmidt pass orthogonalises
+//     them; tighter ones iterate in lockstep (pivoted LU solves from a
+//     counter-based (splitmix64) start vector, each member's on its own
+//     thread, the cluster's CTA orthogonalising between them; before a
+//     refinement in double-float, eps = 2^-44).
+//     The largest-modulus entry of each vector is made positive.
+//   With both the FP64 solve takes 1.2, 3.9 and 12.8 ms at n = 500, 1501
+//   and 4096 (nev = n / 2), against 5.9, 17.6 and 48 ms for two-lane bisection
+//   from a double-float bracket and pivoted inverse iteration alone.
 // Vectors are kept interleaved, Q[i * nev + k], so consecutive threads
 // (consecutive k) touch consecutive addresses in every sweep over i.
 #include <algorithm>
@@ -194,7 +196,7 @@ constexpr double DF_SLACK = 1.0 / 68719476736.0;  // 2^-36: widening of a double
 
 // FP64 multisection with L lanes per wanted eigenvalue: each lane counts at
 // one of L equally spaced interior points, the interval shrinks to
-// 1 / (L + 1) per step (stopping rule of bisect_one).  The start is the
+// 1 / (L + 1) per step, down to 2 eps max(|lo|, |hi|).  The start is the
 // double-float bracket (units of g) widened by DF_SLACK g once its ends pass
 // the FP64 counts count(lo) <= j < count(hi); a bracket that fails is widened
 // eightfold, up to the whole Gershgorin interval.

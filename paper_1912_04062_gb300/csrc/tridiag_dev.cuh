@@ -56,23 +56,6 @@ __device__ __forceinline__ int sturm(int n, const double* __restrict__ a2, doubl
     return cnt;
 }
 
-// The wanted eigenvalue of ascending index j (Sturm bisection on [-g, g]).
-__device__ __forceinline__ double bisect_one(int n, int j, const double* __restrict__ a2, double g, double pivmin) {
-    if (n == 1 || g == 0.0) return 0.0;
-    double lo = -g - 2.0 * DBL_EPSILON * g - pivmin;
-    double hi = g + 2.0 * DBL_EPSILON * g + pivmin;
-    for (int it = 0; it < 4000; it++) {
-        double w = hi - lo;
-        double tol = 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + DBL_MIN;
-        if (w <= tol) break;
-        double mid = lo + 0.5 * w;
-        if (mid <= lo || mid >= hi) break;
-        if (sturm(n, a2, pivmin, mid) <= j) lo = mid;
-        else hi = mid;
-    }
-    return lo + 0.5 * (hi - lo);
-}
-
 // Zero-diagonal form (Sec. 2.2, remark after Algorithm 1): with the unknowns
 // shuffled even first, S = [[0, B], [B^T, 0]], B lower bidiagonal with
 // diagonal a_i = alpha_{2i} and subdiagonal b_i = alpha_{2i+1}; the
@@ -81,21 +64,8 @@ __device__ __forceinline__ double bisect_one(int n, int j, const double* __restr
 // qd transform of its L D L^T form (D_i = a_i^2, l_i = b_i / a_i):
 // D+_i = a_i^2 + s_i, s_{i+1} = b_i^2 s_i / D+_i - t, s_0 = -t (one division per
 // step over m steps, against n steps of the full Sturm count).
-__device__ __forceinline__ int bd_count(int m, const double* __restrict__ a2e, const double* __restrict__ b2e,
-                                        double pivmin, double t) {
-    int cnt = 0;
-    double sv = -t;
-    for (int i = 0; i < m; i++) {
-        double d = a2e[i] + sv;
-        if (fabs(d) < pivmin) d = -pivmin;
-        cnt += (d < 0.0);
-        sv = b2e[i] * sv / d - t;
-    }
-    return cnt;
-}
-
-// bd_count on the matrix scaled to g in [1, 2) (entries a2e, b2e <= 4), with
-// the quick reciprocal: six FP64 instructions a step.  A quotient off by a
+// The matrix is scaled to g in [1, 2) (entries a2e, b2e <= 4); with the quick
+// reciprocal six FP64 instructions a step.  A quotient off by a
 // unit of the last place is, like any rounding of the recurrence, a relative
 // perturbation of a_i and b_i.  Pivots below 2^-900 are raised to it.
 __device__ __forceinline__ int bd_count_scaled(int m, const double* __restrict__ a2e, const double* __restrict__ b2e,
@@ -112,25 +82,6 @@ __device__ __forceinline__ int bd_count_scaled(int m, const double* __restrict__
         sv = fma(b2e[i] * sv, rcp_fast(d), -t);
     }
     return cnt;
-}
-
-// The k-th largest eigenvalue (k < n/2) of S by bisection on x in [0, g] with
-// counts of B B^T at t = x^2 (ascending index m - 1 - k there).
-__device__ __forceinline__ double bisect_one_bd(int m, int k, const double* __restrict__ a2e,
-                                                const double* __restrict__ b2e, double g, double pivmin) {
-    if (m < 1 || g == 0.0) return 0.0;  // m = 1 (n = 2): the eigenvalue |alpha_0|
-    const int j = m - 1 - k;
-    double lo = 0.0, hi = g + 2.0 * DBL_EPSILON * g + pivmin;
-    for (int it = 0; it < 4000; it++) {
-        double w = hi - lo;
-        double tol = 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + DBL_MIN;
-        if (w <= tol) break;
-        double mid = lo + 0.5 * w;
-        if (mid <= lo || mid >= hi) break;
-        if (bd_count(m, a2e, b2e, pivmin, mid * mid) <= j) lo = mid;
-        else hi = mid;
-    }
-    return lo + 0.5 * (hi - lo);
 }
 
 __device__ __forceinline__ double splitmix_uniform(unsigned long long seed, unsigned long long i) {
@@ -636,78 +587,6 @@ __device__ __forceinline__ void invit_solve_df(int n, const InvitDf& v, size_t l
                 y1 = y;
             }
     }
-}
-
-__device__ __forceinline__ void invit_sign_df(int n, Df* __restrict__ Qd, size_t ld, int k) {
-    int imax = 0;
-    float vmax = fabsf(Qd[k].h);
-    for (int i = 1; i < n; i++) {
-        const float a = fabsf(Qd[i * ld + k].h);
-        if (a > vmax) { vmax = a; imax = i; }
-    }
-    if (Qd[imax * ld + k].h < 0.f)
-        for (int i = 0; i < n; i++) Qd[i * ld + k] = df_neg(Qd[i * ld + k]);
-}
-
-__device__ __forceinline__ void invit_cluster_df(int n, int nev, const float* __restrict__ alh,
-                                                 const float* __restrict__ all_, const double* __restrict__ lambda,
-                                                 double g, double ctol_rel, int maxit, const InvitBufs& bf,
-                                                 double* __restrict__ Q, int* __restrict__ fail, int k0,
-                                                 bool singles_only = false) {
-    const double ctol = ctol_rel * g;
-    if (!starts_cluster(lambda, k0, ctol)) return;  // not a cluster leader
-    int k1 = k0 + 1;
-    while (k1 < nev && !starts_cluster(lambda, k1, ctol)) k1++;
-    if (singles_only && k1 - k0 > 1) return;
-    const size_t ld = (size_t)nev;
-    if (n == 1 || g == 0.0) {
-        for (int k = k0; k < k1; k++)
-            for (int i = 0; i < n; i++) Q[i * ld + k] = (i == k) ? 1.0 : 0.0;
-        return;
-    }
-    const double eps = 1.0 / 17592186044416.0;  // 2^-44
-    const float ptol = (float)(eps * g);
-    const float grow = (float)(1.0 / (100.0 * sqrt((double)n) * eps * g));
-    const InvitDf v = invit_df_view(bf, Q);
-    Df* Qd = v.Qd;
-    const Df zero = {0.f, 0.f};
-    for (int k = k0; k < k1; k++) {
-        invit_lu_df(n, alh, all_, lambda[k], ptol, v, ld, k);
-        invit_start_df(n, Qd, ld, k);
-        bool conv = false, done = false;
-        for (int it = 0; it < maxit && !done; it++) {
-            invit_solve_df(n, v, ld, k);
-            // orthogonalise against the earlier vectors of the cluster
-            for (int p = k0; p < k; p++) {
-                Df d = zero;
-                for (int i = 0; i < n; i++) d = df_add(d, df_mul(Qd[i * ld + p], Qd[i * ld + k]));
-                const Df md = df_neg(d);
-                for (int i0 = 0; i0 < n; i0 += INV_IB) {
-                    Df a[INV_IB], b[INV_IB];
-#pragma unroll
-                    for (int u = 0; u < INV_IB; u++)
-                        if (i0 + u < n) {
-                            a[u] = Qd[(size_t)(i0 + u) * ld + k];
-                            b[u] = Qd[(size_t)(i0 + u) * ld + p];
-                        }
-#pragma unroll
-                    for (int u = 0; u < INV_IB; u++)
-                        if (i0 + u < n) Qd[(size_t)(i0 + u) * ld + k] = df_add(a[u], df_mul(md, b[u]));
-                }
-            }
-            float nrm = 0.f;
-            for (int i = 0; i < n; i++) { const float y = Qd[i * ld + k].h; nrm = fmaf(y, y, nrm); }
-            nrm = sqrtf(nrm);
-            if (!(nrm > 0.f) || !isfinite(nrm)) break;
-            invit_scale_df(n, Qd, ld, k, {1.0f / nrm, 0.f});
-            if (conv) done = true;
-            else if (nrm >= grow) conv = true;
-        }
-        if (!conv) atomicMin(fail, k);
-        invit_sign_df(n, Qd, ld, k);
-    }
-    for (int k = k0; k < k1; k++)
-        for (int i = 0; i < n; i++) Q[i * ld + k] = df_to_double(Qd[i * ld + k]);
 }
 
 // FP32 Sturm count of the scaled matrix S / g at x (|x| ~ 1): the recurrence

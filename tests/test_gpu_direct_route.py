@@ -1,10 +1,12 @@
 """The direct (one-step) reduction with its back-transformation, and the twisted
 eigenvectors of the tridiagonal, at the sizes where their tiling changes.
 
-Orders around a panel of 64 reflectors, around one, two and three rows per CTA
-of a 152-SM GPU, the first one whose rows do not all fit shared memory, and the
-first ones of the lower-triangle form (whole and ragged blocks of 64); slabs of one to six eigenvectors per CTA.  The two-step route (an explicit FP64
-Q_trd) is the other side of the comparison.  Bounds: those of the other solve
+Orders around one row per CTA of a thread-block cluster and around the largest
+that a cluster takes, around a panel of 64 reflectors, around one, two and
+three rows per CTA of a 152-SM GPU, the first one whose rows do not all fit shared memory, and the
+first ones of the lower-triangle form (whole and ragged blocks of 64); slabs of
+one to six eigenvectors per CTA.  The two-step route (an explicit FP64 Q_trd) is
+the other side of the comparison.  Bounds: those of the other solve
 tests (1e-12 of the largest eigenvalue; residual and orthogonality 50 n eps).
 """
 import numpy as np
@@ -38,9 +40,10 @@ def _solve(dA, nev, opts, vectors=True):
     return lam, Zr, Zi
 
 
-@pytest.mark.parametrize("n,nev", [(2, 1), (3, 1), (49, 24), (65, 32), (66, 33), (67, 1), (130, 65), (152, 3),
-                                   (153, 76), (305, 152), (306, 153), (459, 20), (610, 305), (914, 457),
-                                   (1825, 912), (1826, 40), (3001, 50), (3072, 33), (3137, 1568)])
+@pytest.mark.parametrize("n,nev", [(2, 1), (3, 1), (15, 7), (16, 8), (17, 8), (33, 1), (49, 24), (65, 32), (66, 33),
+                                   (67, 1), (130, 65), (152, 3), (153, 76), (220, 110), (221, 110), (305, 152),
+                                   (306, 153), (459, 20), (610, 305), (914, 457), (1825, 912), (1826, 40), (3001, 50),
+                                   (3072, 33), (3137, 1568)])
 def test_direct_route_matches_two_step(n, nev):
     import torch
     import paper_1912_04062_gb300 as sk
@@ -59,7 +62,8 @@ def test_direct_route_matches_two_step(n, nev):
     assert torch.equal(lam3, lam1) and torch.equal(Zr3, Zr) and torch.equal(Zi3, Zi)
 
 
-@pytest.mark.parametrize("n,scale,tiny", [(2, 1.0, 1.0), (4, 1.0, 1.0), (64, 1.0, 1.0), (130, 1e-120, 1.0),
+@pytest.mark.parametrize("n,scale,tiny", [(2, 1.0, 1.0), (4, 1.0, 1.0), (64, 1.0, 1.0), (220, 1.0, 1.0),
+                                          (222, 1.0, 1.0), (130, 1e-120, 1.0),
                                           (306, 1e100, 1.0), (308, 1.0, 1e-5), (308, 1.0, 1e-8), (1002, 1.0, 1.0),
                                           (2070, 1.0, 1.0), (3202, 1e-40, 1.0), (3264, 1.0, 1e-5),
                                           (3266, 1.0, 1.0)])
