@@ -43,74 +43,106 @@ __global__ void bse_build_m_kernel(int h, const double* __restrict__ Ar, const d
 
 // Unblocked Cholesky of the kb x kb diagonal block (lower, in place), right
 // looking; a pivot that is not positive and finite records
-// SKEW_ERR_NOT_DEFINITE and stops the factorisation of the block.
+// SKEW_ERR_NOT_DEFINITE and stops the factorisation of the block.  A serial
+// chain of a square root, a quotient (about 600 clocks each) and an update per
+// column: two barriers a column, the roots beside the block so that every
+// thread can test the pivot itself, and the update on thread columns without
+// an integer division.
 __global__ void __launch_bounds__(256) chol_diag_kernel(int kb, double* __restrict__ D, int ld, int* status) {
-    __shared__ double S[CB][CB + 1];
-    __shared__ int bad;
-    const int t = threadIdx.x;
-    for (int e = t; e < kb * kb; e += blockDim.x) {
-        const int i = e % kb, j = e / kb;
-        S[i][j] = (i >= j) ? D[i + (size_t)j * ld] : 0.0;
+    __shared__ double S[CB][CB + 1], root[CB];
+    const int t = threadIdx.x, q = t & (CB - 1);
+    for (int e = t; e < CB * CB; e += 256) {
+        const int i = e % CB, j = e / CB;
+        S[i][j] = (i < kb && i >= j) ? D[i + (size_t)j * ld] : 0.0;
     }
-    if (t == 0) bad = 0;
     __syncthreads();
+    int done = kb;
     for (int j = 0; j < kb; j++) {
-        if (t == 0) {
-            const double d = S[j][j];
-            if (!(d > 0.0) || !isfinite(d)) {
-                bad = 1;
-                sk_set_error(status, SKEW_ERR_NOT_DEFINITE);
-            } else {
-                S[j][j] = sqrt(d);
-            }
+        const double d = S[j][j];
+        if (!(d > 0.0) || !isfinite(d)) {
+            if (t == 0) sk_set_error(status, SKEW_ERR_NOT_DEFINITE);
+            done = j;
+            break;  // every thread reads the same pivot
+        }
+        if (t < CB && t >= j) {
+            const double r = sqrt(d);
+            if (t == j) root[j] = r;
+            else S[t][j] /= r;
         }
         __syncthreads();
-        if (bad) break;
-        const double dj = S[j][j];
-        for (int i = j + 1 + t; i < kb; i += blockDim.x) S[i][j] /= dj;
-        __syncthreads();
-        const int m = kb - j - 1;
-        for (int e = t; e < m * m; e += blockDim.x) {
-            const int i = j + 1 + e % m, l = j + 1 + e / m;
-            if (l <= i) S[i][l] = fma(-S[i][j], S[l][j], S[i][l]);
+        if (q > j) {
+            const double w = S[q][j];
+            for (int i = j + 1 + (t >> 6); i < kb; i += 4)
+                if (q <= i) S[i][q] = fma(-S[i][j], w, S[i][q]);
         }
         __syncthreads();
     }
-    for (int e = t; e < kb * kb; e += blockDim.x) {
-        const int i = e % kb, j = e / kb;
-        if (i >= j) D[i + (size_t)j * ld] = S[i][j];
+    for (int e = t; e < CB * CB; e += 256) {
+        const int i = e % CB, j = e / CB;
+        if (i < kb && i >= j) D[i + (size_t)j * ld] = (i == j && j < done) ? root[j] : S[i][j];
     }
+}
+
+// The two triangular solves with a diagonal block, a warp to each right-hand
+// side (8 to a CTA): lane l holds entries l and l + 32, each step's solution is
+// broadcast by a shuffle and taken off the rest.  64 steps of a short chain,
+// bound by it and by the FP64 pipe of the SMs that have a CTA.  The form with a
+// right-hand side per thread had 64 quotients of 600 clocks in a chain on the
+// few SMs that its CTAs of 128 filled: 139 us a panel and 173 us a block of the
+// back substitution at 2h = 1200 (now 29 and 28), whatever their width.  The
+// driver at h = 600: 29.0 -> 24.7 ms.
+constexpr int TR = 8;
+
+// L (lower, kb x kb at ld) and the reciprocals of its diagonal; zero and one
+// beyond kb, so that the steps there change nothing.
+__device__ inline void load_diag_block(int t, int kb, const double* __restrict__ L, int ld, double (*Ls)[CB + 1],
+                                       double* inv) {
+    for (int e = t; e < CB * CB; e += 256) {
+        const int i = e % CB, j = e / CB;
+        Ls[i][j] = (i < kb && i >= j) ? L[i + (size_t)j * ld] : (i == j ? 1.0 : 0.0);
+    }
+    __syncthreads();
+    if (t < CB) inv[t] = 1.0 / Ls[t][t];
+    __syncthreads();
+}
+
+// s / d from y = 1 / d, corrected once: within an ulp of the quotient
+__device__ __forceinline__ double quot_corrected(double s, double d, double y) {
+    const double x = s * y;
+    return fma(fma(-x, d, s), y, x);
 }
 
 // Panel below a factored diagonal block: P <- P L11^-T (row r: x L11^T = p by
 // forward substitution), and NP = -P for the trailing update's second factor.
-__global__ void __launch_bounds__(128) chol_panel_kernel(int m, int kb, const double* __restrict__ L11, int ld,
+__global__ void __launch_bounds__(256) chol_panel_kernel(int m, int kb, const double* __restrict__ L11, int ld,
                                                          double* __restrict__ P, double* __restrict__ NP, int ldn) {
-    __shared__ double Ls[CB][CB + 1];
-    const int t = threadIdx.x;
-    for (int e = t; e < kb * kb; e += blockDim.x) {
-        const int i = e % kb, j = e / kb;
-        Ls[i][j] = (i >= j) ? L11[i + (size_t)j * ld] : 0.0;
+    __shared__ double Ls[CB][CB + 1], inv[CB], X[TR][CB + 1];
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31, r0 = blockIdx.x * TR;
+    for (int e = t; e < TR * CB; e += 256) {
+        const int r = e % TR, j = e / TR;
+        X[r][j] = (r0 + r < m && j < kb) ? P[r0 + r + (size_t)j * ld] : 0.0;
     }
+    load_diag_block(t, kb, L11, ld, Ls, inv);
+    double a = X[w][lane], b = X[w][lane + 32];
+    for (int j = 0; j < 32; j++) {
+        const double x = quot_corrected(__shfl_sync(~0u, a, j), Ls[j][j], inv[j]);
+        if (lane == j) a = x;
+        if (lane > j) a = fma(-x, Ls[lane][j], a);
+        b = fma(-x, Ls[lane + 32][j], b);
+    }
+    for (int j = 0; j < 32; j++) {
+        const double x = quot_corrected(__shfl_sync(~0u, b, j), Ls[j + 32][j + 32], inv[j + 32]);
+        if (lane == j) b = x;
+        if (lane > j) b = fma(-x, Ls[lane + 32][j + 32], b);
+    }
+    X[w][lane] = a;
+    X[w][lane + 32] = b;
     __syncthreads();
-    const int r = blockIdx.x * blockDim.x + t;
-    if (r >= m) return;
-    double x[CB];
-#pragma unroll
-    for (int j = 0; j < CB; j++) x[j] = (j < kb) ? P[r + (size_t)j * ld] : 0.0;
-#pragma unroll
-    for (int j = 0; j < CB; j++) {
-        if (j < kb) {
-            double s = x[j];
-            for (int l = 0; l < j; l++) s = fma(-x[l], Ls[j][l], s);
-            x[j] = s / Ls[j][j];
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < CB; j++) {
-        if (j < kb) {
-            P[r + (size_t)j * ld] = x[j];
-            NP[r + (size_t)j * ldn] = -x[j];
+    for (int e = t; e < TR * CB; e += 256) {
+        const int r = e % TR, j = e / TR;
+        if (r0 + r < m && j < kb) {
+            P[r0 + r + (size_t)j * ld] = X[r][j];
+            NP[r0 + r + (size_t)j * ldn] = -X[r][j];
         }
     }
 }
@@ -129,33 +161,30 @@ __global__ void bse_jl_kernel(int h, double* __restrict__ L, int ld, double* __r
     }
 }
 
-// Back substitution with one diagonal block: X_I <- L_II^-T X_I, one thread per
+// Back substitution with one diagonal block: X_I <- L_II^-T X_I, a warp per
 // right-hand side column (L_II^T x = z: x_j = (z_j - sum_{l > j} L_lj x_l) / L_jj).
-__global__ void __launch_bounds__(128) trsm_lt_diag_kernel(int kb, const double* __restrict__ Lii, int ld,
+__global__ void __launch_bounds__(256) trsm_lt_diag_kernel(int kb, const double* __restrict__ Lii, int ld,
                                                            double* __restrict__ X, int ldx, int ncols) {
-    __shared__ double Ls[CB][CB + 1];
-    const int t = threadIdx.x;
-    for (int e = t; e < kb * kb; e += blockDim.x) {
-        const int i = e % kb, j = e / kb;
-        Ls[i][j] = (i >= j) ? Lii[i + (size_t)j * ld] : 0.0;
-    }
-    __syncthreads();
-    const int c = blockIdx.x * blockDim.x + t;
+    __shared__ double Ls[CB][CB + 1], inv[CB];
+    const int t = threadIdx.x, lane = t & 31;
+    load_diag_block(t, kb, Lii, ld, Ls, inv);
+    const int c = blockIdx.x * TR + (t >> 5);
     if (c >= ncols) return;
-    double x[CB];
-#pragma unroll
-    for (int j = 0; j < CB; j++) x[j] = (j < kb) ? X[j + (size_t)c * ldx] : 0.0;
-#pragma unroll
-    for (int j = CB - 1; j >= 0; j--) {
-        if (j < kb) {
-            double s = x[j];
-            for (int l = j + 1; l < kb; l++) s = fma(-Ls[l][j], x[l], s);
-            x[j] = s / Ls[j][j];
-        }
+    double* x0 = X + (size_t)c * ldx;
+    double a = (lane < kb) ? x0[lane] : 0.0, b = (lane + 32 < kb) ? x0[lane + 32] : 0.0;
+    for (int j = 31; j >= 0; j--) {
+        const double x = quot_corrected(__shfl_sync(~0u, b, j), Ls[j + 32][j + 32], inv[j + 32]);
+        if (lane == j) b = x;
+        if (lane < j) b = fma(-x, Ls[j + 32][lane + 32], b);
+        a = fma(-x, Ls[j + 32][lane], a);
     }
-#pragma unroll
-    for (int j = 0; j < CB; j++)
-        if (j < kb) X[j + (size_t)c * ldx] = x[j];
+    for (int j = 31; j >= 0; j--) {
+        const double x = quot_corrected(__shfl_sync(~0u, a, j), Ls[j][j], inv[j]);
+        if (lane == j) a = x;
+        if (lane < j) a = fma(-x, Ls[j][lane], a);
+    }
+    if (lane < kb) x0[lane] = a;
+    if (lane + 32 < kb) x0[lane + 32] = b;
 }
 
 // psi = Q x sqrt(lambda), x = Xr + i Xi (2h x nev), Q = [[I, -iI], [I, iI]] / sqrt(2)
@@ -200,7 +229,7 @@ cudaError_t cholesky_lower(cudaStream_t st, int N, double* M, int ld, double* NP
         const int m = N - k0 - kb;
         if (m <= 0) break;
         double* P = D + kb;
-        chol_panel_kernel<<<(m + 127) / 128, 128, 0, st>>>(m, kb, D, ld, P, NP, m);
+        chol_panel_kernel<<<(m + TR - 1) / TR, 256, 0, st>>>(m, kb, D, ld, P, NP, m);
         count_launch();
         // A22 += P (-P)^T on the lower 64-tiles
         if (const cudaError_t e = gemm_lower_tiles(st, m, kb, P, ld, NP, m, D + kb + (size_t)kb * ld, ld, false))
@@ -222,7 +251,8 @@ cudaError_t trsm_lower_t(cudaStream_t st, int N, const double* L, int ld, double
     const int nb = (N + CB - 1) / CB;
     for (int b = nb - 1; b >= 0; b--) {
         const int i0 = b * CB, kb = (N - i0 < CB) ? N - i0 : CB;
-        trsm_lt_diag_kernel<<<(ncols + 127) / 128, 128, 0, st>>>(kb, L + i0 + (size_t)i0 * ld, ld, X + i0, ldx, ncols);
+        trsm_lt_diag_kernel<<<(ncols + TR - 1) / TR, 256, 0, st>>>(kb, L + i0 + (size_t)i0 * ld, ld, X + i0, ldx,
+                                                                    ncols);
         count_launch();
         if (i0 > 0) {
             // X[0:i0, :] -= (L[i0:i0+kb, 0:i0])^T X[i0:i0+kb, :]
