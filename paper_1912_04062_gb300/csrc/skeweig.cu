@@ -1047,7 +1047,7 @@ int skew_eig_profile(int n, const double* A, int lda, int nev, double* lambda, d
 
 namespace {
 struct BseWs {
-    double *M, *JL, *K, *NP;
+    double *M, *Z, *K, *NP;
     int* status;
     void* solve;
     size_t solve_bytes;
@@ -1056,7 +1056,7 @@ bool carve_bse(Carve& cv, int h, int nev, const skew_opts* o, BseWs* w) {
     const size_t N = 2 * (size_t)h;
     w->status = cv.take<int>(16);
     w->M = cv.take<double>(N * N);
-    w->JL = cv.take<double>(N * N);  // J L, later the eigenvectors z of K (N x 2 nev)
+    w->Z = cv.take<double>(2 * N * (size_t)nev);  // the eigenvectors z of K
     w->K = cv.take<double>(N * N);
     w->NP = cv.take<double>(N * 64);
     w->solve_bytes = plan_bytes((int)N, nev, o, true);
@@ -1099,11 +1099,9 @@ int skew_bse_solve(int h, const double* A_re, const double* A_im, int lda, const
     if (const cudaError_t e = bse_build_m(st, h, A_re, A_im, lda, B_re, B_im, ldb, w.M, N)) return cuda_fail(e);
     if (const cudaError_t e = cholesky_lower(st, N, w.M, N, w.NP, w.status)) return cuda_fail(e);
     // 3. K = L^T (J L), then the skew solve (its lower triangle is read)
-    if (const cudaError_t e = bse_jl(st, h, w.M, N, w.JL, N)) return cuda_fail(e);
-    if (const cudaError_t e = gemm(st, true, false, N, N, N, 1.0, w.M, N, w.JL, N, 0.0, w.K, N))
-        return cuda_fail(e);
-    double* Zr = w.JL;
-    double* Zi = w.JL + (size_t)N * nev;
+    if (const cudaError_t e = bse_k(st, h, w.M, N, w.K, N)) return cuda_fail(e);
+    double* Zr = w.Z;
+    double* Zi = w.Z + (size_t)N * nev;
     int rc = run_solve(st, N, w.K, N, nev, lambda, Zr, Zi, N, opts, w.solve, w.solve_bytes, w.status + 1);
     if (rc) return rc;
     // 4. x = L^-T z (real and imaginary parts), psi = Q x sqrt(lambda)
