@@ -14,7 +14,7 @@ region.  ``e2e`` repeats the solve through ``skew_eig_host`` (pinned host
 buffers, host<->device copies inside each call; one warm-up call first).
 ``batched`` (after the main line's own measurements) times the batched
 workload -- 2000 matrices of log-uniform order in [32, 1024], one
-graph-captured persistent launch -- against a loop of single solves.
+graph-captured plan -- against a loop of single solves.
 
 ``cpu_baseline`` times the FP64 CPU oracle on all host cores on a bounded
 sample (the same construction at order --cpu-n, scaled to n by n^3), with
@@ -553,7 +553,7 @@ def run_ours(args, ws, rank, local):
         torch.cuda.empty_cache()
     total_F = 4.0 / 3.0 * n ** 3 + 8.0 * nev * n * n
 
-    # ---- the batched workload (one graph-captured persistent launch against
+    # ---- the batched workload (one graph-captured plan against
     # a loop of single solves), reported beside the main line
     batched = None
     if args.batched_leg > 0:
@@ -615,7 +615,7 @@ def batched_leg(args, ws, rank, local, steps, warmup, loop_warmup=True):
     1024] (odd and even), prescribed spectra l ~ U(0.1, 10), Haar Q, all n/2
     pairs, FP64; under torchrun each rank takes its longest-processing-time
     share (no collective on the data path).  The batch is one plan
-    (skew_batched_plan_*): one persistent launch, captured in a CUDA graph and
+    (skew_batched_plan_*), its launches captured in a CUDA graph and
     replayed; its launch configuration comes from the tuning table for this
     GPU, or is tuned on the batch (--retune, or no entry).  Timed against a
     loop of single solves (skew_eig_ex) on the same device matrices; an
@@ -654,7 +654,7 @@ def batched_leg(args, ws, rank, local, steps, warmup, loop_warmup=True):
     else:
         cfg, source = tuning.lookup(gpu, my_sizes, table), "tuning table"
         plan = sk.BatchedPlan(mats, nevs, config=cfg)
-    # one persistent launch per batch, captured in a CUDA graph
+    # the batch captured in a CUDA graph
     l0 = sk.launch_count()
     side = torch.cuda.Stream()
     side.wait_stream(stream)

@@ -15,9 +15,10 @@
  *
  * Route (all on the device, Algorithm 1): a direct reduction to tridiagonal
  * form (one Householder reflector a column, A <- A + v w^T - w v^T, and the
- * back transformation by those reflectors alone) where it is the faster one,
- * which is up to n of about 4000 to 8000 in the FP64 form and the refined
- * mode; above that, and in the split modes, the two-step form (Sec. 2.1/2.3.2):
+ * back transformation by those reflectors alone) where it is the faster one:
+ * up to n = 16384 in the FP64 form (8000 for values only) and up to 11500 in the
+ * refined mode (5000 for part of the vectors, 4100 for values only); above that,
+ * and in the split modes, the two-step form (Sec. 2.1/2.3.2):
  *   full-to-band (blocked Householder panels, compact WY Q = I - V T V^T,
  *   Eq. 7; skew trailing update A <- A + V W^T - W V^T, Eqs. 8-10 with
  *   U1 = -U2), band-to-tridiagonal bulge chase (Sec. 2.3.2, skew SYR2/SYMV),
@@ -125,8 +126,8 @@ typedef struct {
 
 /* skew_opts.qtrd: arithmetic of the two-step route's Q_trd.  Any value but
  * AUTO keeps the two-step route at every order (except SKEW_QTRD_DF where it is
- * the refined mode's own choice).  SKEW_QTRD_AUTO (0) takes the mode's choice (FP64 in the FP64
- * form; FP32 SIMT when the mixed modes refine; double-float when the refined
+ * the refined mode's own choice).  SKEW_QTRD_AUTO (0) takes the mode's choice
+ * (FP64 in the FP64 form; FP32 SIMT when the mixed modes refine; double-float when the refined
  * mode cannot refine (nev < n/2, odd n) and FP64 in the split modes then);
  * the others force FP32 SIMT, FP64 SIMT, the tensor-core form (compact WY
  * blocks of 64 sweeps, BF16x6 tcgen05 products with FP32 accumulation,

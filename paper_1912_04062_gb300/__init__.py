@@ -530,8 +530,9 @@ def batched_get_config():
 
 
 class BatchedPlan:
-    """A batch of problems (orders <= 1024) prepared once and solved by one
-    persistent launch per execute() (skew_batched_plan_*).  Holds its device
+    """A batch of problems (orders <= 1024) prepared once and solved by a fixed
+    sequence of launches per execute(), each one over all its matrices
+    (skew_batched_plan_*).  Holds its device
     buffers; execute() does no host synchronisation and can be captured in a
     CUDA graph."""
 

@@ -1,8 +1,9 @@
 """Tuned launch configurations of the batched solve, per GPU model.
 
-The batched solve runs as one persistent launch whose two tunables --
-CTAs per SM (1..4) and the largest order kept in shared memory (0..160) --
-trade occupancy against where each working matrix lives.  BatchedPlan.tune()
+The batched solve reduces its matrices of order up to 96 in one persistent
+launch whose two tunables -- CTAs per SM (1..4) and the largest order kept in
+shared memory (0..160) -- trade occupancy against where each working matrix
+lives (larger orders take thread-block clusters, which the library sizes).  BatchedPlan.tune()
 times every candidate on an actual batch; the fastest is recorded here, keyed
 by the GPU's name and by the batch's size class, in ``tuning_table.json``
 next to this file.  ``lookup`` returns the entry of the same size class, else
