@@ -12,11 +12,19 @@
 //   D_k = A[r_k:r_k+L, r_k:r_k+L] (skew) -> H D H = D + v p^T - p v^T with
 //         p = tau D v (the 0.5 tau^2 (v^T D v) v term is 0 for skew D);
 //   C_k = A[r_k+b:r_k+2b, r_k:r_k+L] -> C H (creates the next bulge).
-// Dependencies: step k of sweep s may run once sweep s-1 has finished step
-// k+1 and after step k-1 of its own sweep; the single element it shares with
-// step k+2 of sweep s-1 is completed one step later (see chase_task).
+// Dependencies: step k of sweep s may run after step k-1 of its own sweep and
+// once sweep s-1 has stored B_{k+1} and the first column of D_{k+1} (the rows
+// and columns of D_k and C_k of sweep s lie one further down, so nothing else
+// of step k+1 is among them); the single element it shares with step k+2 of
+// sweep s-1 is completed one step later (see chase_task).
 // One persistent cooperative launch: CTA g owns sweeps g, g+G, ...; a per-sweep
-// progress counter (release store / acquire load, capped spin) orders them.
+// progress counter (release store / acquire load, capped spin) orders them: it
+// stands at 2k+1 once step k has stored B_k and the first column of D_k, and at
+// 2k+2 after the whole step.  Bound by the chain of steps, n times (a whole step
+// plus the part of one before its first release), and a step by the FP64 pipe
+// of its SM (766 warp FMAs, 19 clocks each); the first release lets the next
+// sweep start before the C product and the updates of C and D.  n = 6001: the
+// solve with a tenth of the vectors 359.6 -> 351.7 ms, the same bits.
 #include "common.cuh"
 #include "internal.h"
 
@@ -106,6 +114,33 @@ __device__ __forceinline__ bool chase_lower(int t, int u, int& i, int& j) {
     return p < 31;
 }
 
+// One of the products of a step (w = warp / 4: tau v^T B, tau D v, tau C v), 16
+// columns a warp.
+__device__ __forceinline__ void chase_product(int warp, const double* __restrict__ B, const double* __restrict__ D,
+                                              const double* __restrict__ C, ChaseSmem& sm) {
+    const int lane = threadIdx.x & 31, h = lane >> 4, col = 16 * (warp & 3) + (lane & 15), which = warp >> 2;
+    const double* vr = sm.v + 32 * h;
+    double a0 = 0.0, a1 = 0.0;
+    if (which == 0) {
+        const double* x = B + col * CLD + 32 * h;
+#pragma unroll 8
+        for (int e = 0; e < 32; e += 2) {
+            a0 = fma(vr[e], x[e], a0);
+            a1 = fma(vr[e + 1], x[e + 1], a1);
+        }
+    } else {
+        const double* x = ((which == 1) ? D : C) + 32 * h * CLD + col;
+#pragma unroll 8
+        for (int e = 0; e < 32; e += 2) {
+            a0 = fma(x[e * CLD], vr[e], a0);
+            a1 = fma(x[(e + 1) * CLD], vr[e + 1], a1);
+        }
+    }
+    double a = a0 + a1;
+    a += __shfl_down_sync(0xffffffffu, a, 16);
+    if (h == 0) (which == 0 ? sm.wB : (which == 1 ? sm.wD : sm.wC))[col] = sm.tau * a;
+}
+
 // Step k of sweep s.  B holds B_k already when have_b (it is the C block of
 // step k-1 of the same sweep), so its reflector is formed while the previous
 // sweep's progress is awaited; C is kept for step k+1 instead of being stored
@@ -114,7 +149,10 @@ __device__ __forceinline__ bool chase_lower(int t, int u, int& i, int& j) {
 // (0, .., 0, E) before step k: with defer_e, row 63 of C_k is left at zero
 // and step k+1 (fix_e) completes it from the final E as
 // E e_63^T - (tau (E v_63)) v^T, the same operations the full update takes,
-// so a sweep need only wait for step k+1 of its predecessor.  The work is bound by the
+// so a sweep need only wait for (the first release of) step k+1 of its
+// predecessor; without defer_e, at the lower end of the band, E is the element
+// that the predecessor's last step stores with its C, and the wait is for the
+// whole step.  The work is bound by the
 // FP64 pipe (2 FMA per clock per SM): every FP64 warp instruction is spent on
 // needed elements, and the 3 x 64 matrix-vector products take two threads
 // each (rows split between the half-warps) with a single combining add.
@@ -126,7 +164,7 @@ __device__ bool chase_task(int n, int s, int k, int nsw, const int* __restrict__
                            double* __restrict__ Vtrd, double* __restrict__ tautrd, float* __restrict__ V32,
                            float* __restrict__ tau32, int nsw64, double* __restrict__ B, double* __restrict__ D,
                            double* __restrict__ C, bool have_b, bool keep_c, bool fix_e, bool defer_e,
-                           ChaseSmem& sm, unsigned spin_cap) {
+                           ChaseSmem& sm, unsigned spin_cap, int* __restrict__ prog_mine) {
     const int t = threadIdx.x, warp = t >> 5;
     const int r = s + 1 + k * CB;
     const int L = min(CB, n - r);
@@ -213,69 +251,60 @@ __device__ bool chase_task(int n, int s, int k, int nsw, const int* __restrict__
     for (int u = 0; u < CH_EPT; u++) C[(q + CH_JS * u) * CLD + i] = c[u];
     __syncthreads();
 
-    // ---- (v^T B)_col, (D v)_col, (C v)_col on warps 0..11: warp w takes
-    // product w/4 for columns 16 (w mod 4) + 0..15, lanes 16..31 the rows
-    // 32..63 of the lanes 0..15; two accumulators per thread keep the FP64
-    // pipe fed.  Step 0 has no B product.
-    if (warp < 12 && (have_b || warp >= 4)) {
-        const int lane = t & 31, h = lane >> 4, col = 16 * (warp & 3) + (lane & 15), which = warp >> 2;
-        const double* vr = sm.v + 32 * h;
-        double a0 = 0.0, a1 = 0.0;
-        if (which == 0) {
-            const double* x = B + col * CLD + 32 * h;
-#pragma unroll 8
-            for (int e = 0; e < 32; e += 2) {
-                a0 = fma(vr[e], x[e], a0);
-                a1 = fma(vr[e + 1], x[e + 1], a1);
-            }
-        } else {
-            const double* x = ((which == 1) ? D : C) + 32 * h * CLD + col;
-#pragma unroll 8
-            for (int e = 0; e < 32; e += 2) {
-                a0 = fma(x[e * CLD], vr[e], a0);
-                a1 = fma(x[(e + 1) * CLD], vr[e + 1], a1);
-            }
-        }
-        double a = a0 + a1;
-        a += __shfl_down_sync(0xffffffffu, a, 16);
-        if (h == 0) (which == 0 ? sm.wB : (which == 1 ? sm.wD : sm.wC))[col] = sm.tau * a;
-    }
+    // ---- (v^T B)_col and (D v)_col on warps 0..7: warp w takes product w/4
+    // for columns 16 (w mod 4) + 0..15, lanes 16..31 the rows 32..63 of the
+    // lanes 0..15; two accumulators per thread keep the FP64 pipe fed.  Step 0
+    // has no B product.
+    if (warp < 8 && (have_b || warp >= 4)) chase_product(warp, B, D, C, sm);
     __syncthreads();
 
-    // ---- updates, straight to memory: B[:, 1:] -= v wB^T and B[:, 0] =
-    // beta e1; D += v p^T - p v^T with p = wD = tau D v (the 1/2 tau^2
-    // (v^T D v) v term is 0 for skew D); C -= wC v^T (kept as the next B)
-    {
-        const double vi = sm.v[i], wCi = sm.wC[i], beta = sm.beta;
+    // ---- what the next sweep waits for, straight to memory: B[:, 1:] -= v
+    // wB^T and B[:, 0] = beta e1; column 0 of D += v p^T - p v^T with p = wD =
+    // tau D v (the 1/2 tau^2 (v^T D v) v term is 0 for skew D)
+    const double vi = sm.v[i], beta = sm.beta;
 #pragma unroll
-        for (int u = 0; u < CH_EPT; u++) {
-            const int j = q + CH_JS * u;
-            const double vj = sm.v[j];
-            if (i < L) {
-                if (have_b) {
-                    const double bv = (j == 0) ? ((i == 0) ? beta : 0.0) : fma(-vi, sm.wB[j], B[j * CLD + i]);
-                    AB[(size_t)(r - CB + j) * ldab + (CB + i - j)] = bv;
-                } else if (j == 0) {
-                    AB[(size_t)s * ldab + (r - s + i)] = (i == 0) ? beta : 0.0;
-                }
+    for (int u = 0; u < CH_EPT; u++) {
+        const int j = q + CH_JS * u;
+        if (i < L) {
+            if (have_b) {
+                const double bv = (j == 0) ? ((i == 0) ? beta : 0.0) : fma(-vi, sm.wB[j], B[j * CLD + i]);
+                AB[(size_t)(r - CB + j) * ldab + (CB + i - j)] = bv;
+            } else if (j == 0) {
+                AB[(size_t)s * ldab + (r - s + i)] = (i == 0) ? beta : 0.0;
             }
-            const bool inc = i < Lc && j < L;
-            const double cv = inc ? fma(-wCi, vj, c[u]) : 0.0;
-            if (keep_c)
-                C[j * CLD + i] = cv;
-            else if (inc)
-                AB[(size_t)(r + j) * ldab + (CB + i - j)] = cv;
         }
-        if (defer_e && t < CB) {
-            sm.vprev[t] = sm.v[t];
-            if (t == 0) sm.tauprev = sm.tau;
-        }
+    }
+    // threads 0..62 hold column 0 of D in d[0]
+    if (t < CB - 1 && dv[0])
+        AB[(size_t)r * ldab + di[0]] = fma(-sm.wD[di[0]], sm.v[0], fma(sm.v[di[0]], sm.wD[0], d[0]));
+    // all stores precede the release (bar.sync, then a gpu-scope release by one
+    // thread)
+    __syncthreads();
+    if (t == 0) sk_st_release_s32(prog_mine, 2 * k + 1);
+
+    // ---- (C v)_col, then C -= wC v^T (kept as the next B) and the rest of D
+    if (warp >= 8 && warp < 12) chase_product(warp, B, D, C, sm);
+    __syncthreads();
+    const double wCi = sm.wC[i];
 #pragma unroll
-        for (int u = 0; u < 2; u++) {
-            if (dv[u]) {
-                const int ii = di[u], jj = dj[u];
-                AB[(size_t)(r + jj) * ldab + (ii - jj)] = fma(-sm.wD[ii], sm.v[jj], fma(sm.v[ii], sm.wD[jj], d[u]));
-            }
+    for (int u = 0; u < CH_EPT; u++) {
+        const int j = q + CH_JS * u;
+        const bool inc = i < Lc && j < L;
+        const double cv = inc ? fma(-wCi, sm.v[j], c[u]) : 0.0;
+        if (keep_c)
+            C[j * CLD + i] = cv;
+        else if (inc)
+            AB[(size_t)(r + j) * ldab + (CB + i - j)] = cv;
+    }
+    if (defer_e && t < CB) {
+        sm.vprev[t] = sm.v[t];
+        if (t == 0) sm.tauprev = sm.tau;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+        if (dv[u] && (u > 0 || t >= CB - 1)) {
+            const int ii = di[u], jj = dj[u];
+            AB[(size_t)(r + jj) * ldab + (ii - jj)] = fma(-sm.wD[ii], sm.v[jj], fma(sm.v[ii], sm.wD[jj], d[u]));
         }
     }
     return true;
@@ -297,17 +326,16 @@ chase_kernel(int n, double* __restrict__ AB, int ldab, double* __restrict__ alph
         bool have_b = false, fix_e = false;
         for (int k = 0; k < ns; k++) {
             const bool keep_c = k + 1 < ns;  // step k+1 starts from this C
-            // steps 0..k+1 of sweep s-1 done; E of C_k is final only after
-            // its step k+2 (when that exists), awaited by step k+1
-            const int want = (s > 0) ? min(k + 2, nsp) : 0;
+            // steps 0..k of sweep s-1 done and step k+1 at its first release
+            // (all of it without defer_e); E of C_k is final only after its
+            // step k+2 (when that exists), awaited by step k+1
             const bool defer_e = s > 0 && n - (s + 1 + k * CB) >= 2 * CB && k + 2 < nsp;
+            const int want = (s > 0) ? (defer_e ? 2 * k + 3 : 2 * min(k + 2, nsp)) : 0;
             if (!chase_task(n, s, k, nsw, prog + (s > 0 ? s - 1 : 0), want, status, AB, ldab, alpha, Vtrd, tautrd,
-                            V32, tau32, nsw64, B, D, C, have_b, keep_c, fix_e, defer_e, sm, spin_cap))
+                            V32, tau32, nsw64, B, D, C, have_b, keep_c, fix_e, defer_e, sm, spin_cap, prog + s))
                 return;
-            // all stores of the step precede the release (bar.sync, then a
-            // gpu-scope release by one thread)
             __syncthreads();
-            if (threadIdx.x == 0) sk_st_release_s32(prog + s, k + 1);
+            if (threadIdx.x == 0) sk_st_release_s32(prog + s, 2 * k + 2);
             double* tmp = B;  // C_k is B_{k+1}
             B = C;
             C = tmp;
