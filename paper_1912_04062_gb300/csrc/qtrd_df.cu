@@ -12,13 +12,14 @@
 //
 // Structure (the FP32 sliding-window kernel's): reflectors grouped into
 // blocks of 64 sweeps x one step (a parallelogram of rows top .. top+126);
-// each CTA owns a slab of columns, eight threads per column (row phase q), and
+// each CTA owns a slab of columns, P threads per column (row phase q), and
 // keeps the block's window in registers; consecutive blocks of a group share
 // 63 rows, so the window slides by 64 rows, the 64 new rows arriving by
 // cp.async while the block computes.  The FP64 reflectors of the next block
 // arrive by one bulk copy and are split into hi / lo pairs in place.
 //
-// Register window.  Thread q holds window rows 8u + q (u < 16).  The
+// Register window (for P = 8; 16 has half the rows and elements a thread).
+// Thread q holds window rows 8u + q (u < 16).  The
 // reflector at offset off = 8m + r (r = off mod 8) touches rows off .. off+63,
 // that is for this thread the rows 8(m + w) + q with w = 1..7 always, plus
 // w = 0 when q >= r or w = 8 when q < r: exactly 8 elements.  The registers
@@ -26,8 +27,16 @@
 // register index is a compile-time constant for all eight reflectors of one
 // m (r only moves shared-memory offsets, so they run as a loop, keeping the
 // code small), and one rotation by a register between consecutive m keeps
-// the invariant.  Eight threads per column give twice the warps of four, so
-// the four schedulers of an SM get near-equal shares of a slab.
+// the invariant.
+//
+// Threads per column.  A reflector is a chain: the thread's terms, log2 P
+// shuffle levels, the update.  With few columns an SM (a tenth of the vectors
+// of n = 6001: 8) the chain and the idle schedulers bound it, and 16 threads a
+// column halve the terms and fill all four schedulers; with many, the issue
+// rate does, and 8 threads spend one shuffle level less.  n = 4096, 8 against
+// 16 threads: 51.4 / 39.8 ms up to 8 columns a CTA, 48.8 / 46.7 at 12, 47.5 /
+// 46.0 at 16, 62.2 / 55.4 at 24, 61.6 / 66.3 at 32.  The n = 6001 solve
+// 351.7 -> 326.6 ms.
 #include "common.cuh"
 #include "internal.h"
 #include "sm100.cuh"
@@ -38,11 +47,9 @@ namespace {
 constexpr int DB = 64;              // band width = reflector length
 constexpr int DELL = 64;            // sweeps per block
 constexpr int DH = DELL + DB - 1;   // window height
-constexpr int P = 8;                // threads per column (row phases)
-constexpr int NR = 128 / P;         // window rows per thread
-constexpr int MS = DELL / P;        // rotation steps per block
 constexpr int DLD = 72;             // staging leading dimension in doubles (conflict-free halves)
-constexpr int QD_MAXT = 512;        // threads per CTA at most (64 columns)
+constexpr int QD_MAXT = 512;        // threads per CTA at most (64 columns of 8)
+constexpr int WIDE_SLAB = 24;       // columns of a CTA up to which 16 threads take one
 
 __host__ __device__ inline int df_qsteps(int n, int s) { return (s <= n - 3) ? 1 + (n - 3 - s) / DB : 0; }
 
@@ -127,19 +134,21 @@ struct DfSmem {
 
 // One reflector at offset off = P m + r of the block: vb points at its element
 // 0 (hi, lo pairs), H / L registers in the rotated layout of m.  Thread q's
-// elements are i = P w + q - r for w = 1..7 and the edge w = 0 (q >= r) or
-// w = 8 (q < r); every register index is a compile-time constant, r and q
+// elements are i = P w + q - r for w = 1..NE-1 and the edge w = 0 (q >= r) or
+// w = NE (q < r); every register index is a compile-time constant, r and q
 // only move the shared-memory offsets and pick the edge register.
-SK_DEV void df_reflector(float (&H)[NR], float (&L)[NR], const float2* __restrict__ vb, float2 tau, int q, int r) {
+template <int P>
+SK_DEV void df_reflector(float (&H)[128 / P], float (&L)[128 / P], const float2* __restrict__ vb, float2 tau, int q, int r) {
+    constexpr int NE = DB / P;  // elements of a thread
     if (tau.x == 0.f) return;  // absent step or zero tail: H = I
     const bool low = q >= r;
     const float2 ve = vb[low ? q - r : DB + q - r];
-    const float2* vw = vb + P + q - r;  // vw[P (w - 1)] = element P w + q - r, w = 1..7
-    const float eh0 = low ? H[0] : H[P], el0 = low ? L[0] : L[P];
+    const float2* vw = vb + P + q - r;  // vw[P (w - 1)] = element P w + q - r, w = 1..NE-1
+    const float eh0 = low ? H[0] : H[NE], el0 = low ? L[0] : L[NE];
     float S0 = 0.f, C0 = 0.f, S1 = 0.f, C1 = 0.f;
     dot_term(ve.x, ve.y, eh0, el0, S0, C0);
 #pragma unroll
-    for (int w = 1; w < P; w++) {
+    for (int w = 1; w < NE; w++) {
         const float2 v = vw[P * (w - 1)];
         if (w & 1) dot_term(v.x, v.y, H[w], L[w], S1, C1);
         else dot_term(v.x, v.y, H[w], L[w], S0, C0);
@@ -163,21 +172,24 @@ SK_DEV void df_reflector(float (&H)[NR], float (&L)[NR], const float2* __restric
         H[0] = eh;
         L[0] = el;
     } else {
-        H[P] = eh;
-        L[P] = el;
+        H[NE] = eh;
+        L[NE] = el;
     }
 #pragma unroll
-    for (int w = 1; w < P; w++) {
+    for (int w = 1; w < NE; w++) {
         const float2 v = vw[P * (w - 1)];
         axpy_term(ah, al, v.x, v.y, H[w], L[w]);
     }
 }
 
+template <int P>
 __global__ void __launch_bounds__(QD_MAXT, 1)
 qtrd_df_kernel(int n, const double* __restrict__ Vtrd, const double* __restrict__ tautrd, double* __restrict__ Z,
                int ldz, int ncols, int slab, int* status) {
     extern __shared__ __align__(128) unsigned char qd_raw[];
     DfSmem& sm = *reinterpret_cast<DfSmem*>(qd_raw);
+    constexpr int NR = 128 / P;   // window rows per thread
+    constexpr int MS = DELL / P;  // rotation steps per block
     const int nsw = n - 2;
     const int c0 = blockIdx.x * slab;
     const int nc = min(slab, ncols - c0);
@@ -270,11 +282,11 @@ qtrd_df_kernel(int n, const double* __restrict__ Vtrd, const double* __restrict_
 #pragma unroll 1
                 for (int r = P - 1; r >= 0; r--) {
                     const int off = P * m + r;
-                    df_reflector(H, L, vblk + (size_t)off * DB, sm.tau[buf][off], q, r);
+                    df_reflector<P>(H, L, vblk + (size_t)off * DB, sm.tau[buf][off], q, r);
                 }
-                // renormalise the pairs these P reflectors touched (w = 0..P)
+                // renormalise the pairs these P reflectors touched (w = 0..DB/P)
 #pragma unroll
-                for (int w = 0; w <= P; w++) {
+                for (int w = 0; w <= DB / P; w++) {
                     float s, e;
                     two_sum(H[w], L[w], s, e);
                     H[w] = s;
@@ -351,6 +363,21 @@ qtrd_df_kernel(int n, const double* __restrict__ Vtrd, const double* __restrict_
 
 }  // namespace
 
+template <int P>
+static cudaError_t launch_qtrd_df(cudaStream_t st, int n, const double* Vtrd, const double* tautrd, double* Z, int ldz,
+                                  int k, int slab, int* status) {
+    // at least 64 threads: thread t < 64 brings the tau of sweep t
+    const int grid = (k + slab - 1) / slab, threads = max(64, (P * slab + 31) / 32 * 32);
+    const size_t smem = sizeof(DfSmem);
+    if (const cudaError_t e =
+            cudaFuncSetAttribute(qtrd_df_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
+        return e;
+    KtScope kt(st, KT_QTRD);
+    qtrd_df_kernel<P><<<grid, threads, smem, st>>>(n, Vtrd, tautrd, Z, ldz, k, slab, status);
+    count_launch();
+    return cudaGetLastError();
+}
+
 cudaError_t apply_qtrd_df(cudaStream_t st, int n, int b, const double* Vtrd, const double* tautrd, double* Z,
                           int ldz, int k, int* status) {
     if (b != DB) return cudaErrorInvalidValue;
@@ -358,7 +385,7 @@ cudaError_t apply_qtrd_df(cudaStream_t st, int n, int b, const double* Vtrd, con
     // one CTA per SM (the staging takes 140 KB); slabs of at most 64 columns
     // sized so that the CTAs fill whole waves
     const int sms = device_sms();
-    const int maxslab = QD_MAXT / P;
+    const int maxslab = QD_MAXT / 8;
     int waves = 1, slab = maxslab;
     while (true) {
         slab = (k + sms * waves - 1) / (sms * waves);
@@ -366,15 +393,8 @@ cudaError_t apply_qtrd_df(cudaStream_t st, int n, int b, const double* Vtrd, con
         waves++;
     }
     if (slab < 8) slab = (k < 8) ? k : 8;
-    const int grid = (k + slab - 1) / slab;
-    // at least 64 threads: thread t < 64 brings the tau of sweep t
-    const int threads = max(64, (P * slab + 31) / 32 * 32);
-    const size_t smem = sizeof(DfSmem);
-    cudaFuncSetAttribute(qtrd_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    KtScope kt(st, KT_QTRD);
-    qtrd_df_kernel<<<grid, threads, smem, st>>>(n, Vtrd, tautrd, Z, ldz, k, slab, status);
-    count_launch();
-    return cudaGetLastError();
+    return slab <= WIDE_SLAB ? launch_qtrd_df<16>(st, n, Vtrd, tautrd, Z, ldz, k, slab, status)
+                             : launch_qtrd_df<8>(st, n, Vtrd, tautrd, Z, ldz, k, slab, status);
 }
 
 }  // namespace sk

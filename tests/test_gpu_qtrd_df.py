@@ -154,3 +154,24 @@ def test_refined_partial_solve_with_df_qtrd_matches_oracle(n, nev):
     for j in np.flatnonzero(gap > 1e-3 * lam_o[0])[:20]:
         ov = abs(np.vdot(Qo[:, j], Z[:, j]))
         assert abs(ov - 1.0) <= 1e-9, (j, ov)
+
+
+@pytest.mark.parametrize("per_sm,extra", [(8, 1), (16, 3), (24, 0), (24, 1), (33, 0)])
+def test_qtrd_df_threads_per_column(per_sm, extra):
+    # around the widths where a column changes from 16 threads to 8 (24 columns
+    # an SM) and where the slabs are ragged; reflectors past the last sweep
+    import torch
+    import paper_1912_04062_gb300 as sk
+    n = 195
+    k = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    Vtrd, tau, rng = _chase(n, 8500)
+    Z0 = rng.standard_normal((n, k))
+    Zref = sk.fortran(torch.from_numpy(Z0).cuda())
+    sk.apply_qtrd(Vtrd, tau, Zref)
+    Z = sk.fortran(torch.from_numpy(Z0).cuda())
+    st = sk.apply_qtrd_df(Vtrd, tau, Z)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    ref, out = Zref.cpu().numpy(), Z.cpu().numpy()
+    col = np.linalg.norm(out - ref, axis=0) / np.linalg.norm(ref, axis=0)
+    assert np.max(col) <= 32 * 2.0 ** -46 * np.sqrt(n)
