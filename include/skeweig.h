@@ -17,7 +17,7 @@
  * form (one Householder reflector a column, A <- A + v w^T - w v^T, and the
  * back transformation by those reflectors alone) where it is the faster one:
  * up to n = 16384 in the FP64 form (8000 for values only) and up to 11500 in the
- * refined mode (5000 for part of the vectors, 4100 for values only); above that,
+ * refined mode (4750 for part of the vectors, 4000 for values only); above that,
  * and in the split modes, the two-step form (Sec. 2.1/2.3.2):
  *   full-to-band (blocked Householder panels, compact WY Q = I - V T V^T,
  *   Eq. 7; skew trailing update A <- A + V W^T - W V^T, Eqs. 8-10 with

@@ -113,10 +113,11 @@ struct Plan {
 // FP64 values only: the reduction against band reduction and chase (8192: 974
 // against 977 ms, 4000: 134 against 228).  Refined: 8192 0.50 s against 0.75 s,
 // 12288 1.78 against 1.82, 16384 3.98 against 3.61; partial vectors take the FP64
-// form against products of 8 slices (5000: equal; 6001: 400 against 332 ms with
-// the chase and Q_trd), as do values only (4000: 146 against 147 ms).
-constexpr int ONESTEP_FP64 = 16384, ONESTEP_FP64_VALUES = 8000, ONESTEP_REFINE = 11500, ONESTEP_PARTIAL = 5000,
-              ONESTEP_VALUES = 4100;
+// form against products of 8 slices, chase and double-float Q_trd (a tenth or a
+// fiftieth of them: 4200 169 against 201 ms, 4600 208 / 226, 5000 274 / 254), as
+// do values only (3600 112 / 126, 4100 153 / 146).
+constexpr int ONESTEP_FP64 = 16384, ONESTEP_FP64_VALUES = 8000, ONESTEP_REFINE = 11500, ONESTEP_PARTIAL = 4750,
+              ONESTEP_VALUES = 4000;
 // Orders above which the direct reduction keeps the lower triangle only: FP64
 // 3002 67 against 67 ms, 4096 139 against 152; pairs 3002 37.6 against 35.0,
 // 4096 63 against 84.
