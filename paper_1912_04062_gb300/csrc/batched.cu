@@ -231,6 +231,8 @@ SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, do
     __shared__ double2 s_coef[CMAXR];  // sigma u_i, -sigma p_i of the own rows
     __shared__ double s_red[4];
     __shared__ double s_sc[4];
+    __shared__ unsigned long long s_amax[16];  // max |A| over each CTA's rows
+    __shared__ unsigned long long s_wmax[CT / 32];
     const int G = (int)cl_size(), g = (int)cl_rank();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int ldn = cl_ld(n);
@@ -244,6 +246,7 @@ SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, do
     const int rs0 = Rt > srows ? Rt - srows : 0, ilast = g + (Rt - 1) * G;
     // own rows of the full skew matrix: -A(j, i) right of the diagonal
     // (contiguous), A(i, j) left of it
+    unsigned long long am = 0;
     for (int r = 0; r < Rt; r++) {
         const int i = g + r * G;
         double* row = r >= rs0 ? rows + (size_t)(r - rs0) * ldn : S + (size_t)i * n;
@@ -251,7 +254,18 @@ SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, do
             const double v = j > i ? -A[(size_t)i * lda + j] : j < i ? A[(size_t)j * lda + i] : 0.0;
             if (check && !isfinite(v)) sk_set_error(status, SKEW_ERR_NONFINITE);
             row[j] = v;
+            const unsigned long long b = os_abs_bits(v);
+            am = b > am ? b : am;
         }
+    }
+    am = os_warp_max(am);
+    if (lane == 0) s_wmax[warp] = am;
+    __syncthreads();
+    if (warp == 0) {
+        am = os_warp_max(lane < CT / 32 ? s_wmax[lane] : 0ull);
+        if (lane < G)
+            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(cl_map(s_amax + g, (uint32_t)lane)), "l"(am)
+                         : "memory");
     }
     // zeros of V above the reflectors and in the columns that fill up the
     // last panel (the values come after the first barrier below)
@@ -262,6 +276,16 @@ SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, do
     }
     if (g == 0)
         for (int c = n - 2 + t; c < vc; c += CT) tau[c] = 0.0;
+    cl_barrier();
+    am = 0;
+    for (int c = 0; c < G; c++) am = s_amax[c] > am ? s_amax[c] : am;
+    const double scale = os_scale(am);
+    if (scale != 1.0) {
+        for (int r = 0; r < Rt; r++) {
+            double* row = r >= rs0 ? rows + (size_t)(r - rs0) * ldn : S + (size_t)(g + r * G) * n;
+            for (int j = t; j < n; j += CT) row[j] *= scale;
+        }
+    }
     double beta = 0.0, sigma = 0.0;
     for (int k = 0; k + 1 < n; k++) {
         const bool act = ilast > k;  // rows left
@@ -270,7 +294,7 @@ SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, do
             const double2* in = qa + (size_t)(k & 1) * n;
             if (k == 0) {
                 for (int j = t; j < n; j += CT) {
-                    x[j] = j > 0 ? A[j] : 0.0;
+                    x[j] = j > 0 ? scale * A[j] : 0.0;
                     u[j] = 0.0;
                     p[j] = 0.0;
                 }
@@ -324,7 +348,7 @@ SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, do
                 const double s2 = (s_red[0] + s_red[1]) + (s_red[2] + s_red[3]);
                 const double x0 = x[k + 1];
                 double b = x0, sg = 0.0, inv = 0.0;
-                if (s2 != 0.0) {
+                if (os_tail(s2)) {
                     const double rr = sqrt(fma(x0, x0, s2));
                     b = (x0 >= 0.0) ? -rr : rr;
                     // this chain is the longest of a column at small orders
@@ -357,6 +381,10 @@ SK_DEV void cluster_reduce_body(int n, const double* __restrict__ A, int lda, do
             x = sw;
         }
         __syncthreads();
+    }
+    if (scale != 1.0 && ilast == n - 1) {  // this CTA has written every entry
+        __syncthreads();
+        for (int j = t; j < n - 1; j += CT) alpha[j] /= scale;
     }
 }
 

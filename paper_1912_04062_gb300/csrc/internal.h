@@ -64,8 +64,10 @@ cudaError_t tfactor_panels(cudaStream_t st, int panels, const double* tau, const
 size_t onestep_ws(int n);
 // Columns of V (and entries of tau): n - 2 rounded up to whole panels of 64.
 int onestep_vcols(int n);
-// Full skew matrix by rows (F[i * n + j]) from the strict lower triangle of A.
-cudaError_t onestep_full(cudaStream_t st, int n, const double* A, int lda, double* F, int check, int* status);
+// Full skew matrix by rows (F[i * n + j]) from the strict lower triangle of A;
+// ws is that of onestep_reduce (its counter and max |A| are set here).
+int onestep_full(cudaStream_t st, int n, const double* A, int lda, double* F, int check, void* ws, size_t ws_bytes,
+                 int* status);
 // F (overwritten) -> alpha (T[c, c + 1], n - 1), V (n x onestep_vcols, ld n:
 // column k is reflector k, zero above row k + 1, one there) and tau.  spin_cap
 // as in band_reduce.

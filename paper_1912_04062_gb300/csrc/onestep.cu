@@ -51,7 +51,8 @@ struct OsArgs {
     double* tau;   // n entries
     double* alpha; // T[k, k + 1]
     double2* qa;   // 2 n: (q, a), double-buffered
-    unsigned* ctr; // arrivals (zeroed by the caller)
+    unsigned* ctr; // arrivals, zeroed by onestep_full
+    const unsigned long long* amax;  // max |A| (os_scale)
     int* status;
     unsigned cap;
     int srows;     // own rows kept in shared memory (the last ones: they live longest)
@@ -74,8 +75,12 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
     const int Rt = (n - 1 - g) / G + 1;              // own rows: g, g + G, ...
     const int rs0 = Rt > o.srows ? Rt - o.srows : 0; // the first one in shared memory
     const int ilast = g + (Rt - 1) * G;
+    const double scale = os_scale(*o.amax);
     for (int r = rs0; r < Rt; r++)
-        for (int j = t; j < n; j += OT) rows[(size_t)(r - rs0) * ldn + j] = o.F[(size_t)(g + r * G) * n + j];
+        for (int j = t; j < n; j += OT) rows[(size_t)(r - rs0) * ldn + j] = scale * o.F[(size_t)(g + r * G) * n + j];
+    if (scale != 1.0)  // row 0 is read by all below, and never again
+        for (int r = g == 0 ? 1 : 0; r < rs0; r++)
+            for (int j = t; j < n; j += OT) o.F[(size_t)(g + r * G) * n + j] *= scale;
     unsigned target = 0;
     double beta = 0.0, sigma = 0.0;
     for (int k = 0; k + 1 < n; k++) {
@@ -85,7 +90,7 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
         if (k == 0) {
             // column 0 of A, nothing pending: element (j, 0) = -element (0, j)
             for (int j = t; j < n; j += OT) {
-                x[j] = -o.F[j];
+                x[j] = -scale * o.F[j];
                 u[j] = 0.0;
                 p[j] = 0.0;
             }
@@ -119,7 +124,7 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
         if (k == n - 2) {
             // T[n-1, n-2] = x_{n-1}; this CTA owns the last row
             if (t == 0) o.alpha[k] = -x[n - 1];
-            return;
+            break;
         }
         // ---- 2. update the own rows i > k and multiply by x
         const int rf = (k + 1 > g) ? (k + 1 - g + G - 1) / G : 0;  // first own row below k
@@ -171,7 +176,7 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
                 const double s2 = (s_red[0] + s_red[1]) + (s_red[2] + s_red[3]);
                 const double x0 = x[k + 1];
                 double b = x0, sg = 0.0, inv = 0.0;
-                if (s2 != 0.0) {
+                if (os_tail(s2)) {
                     const double rr = sqrt(fma(x0, x0, s2));
                     b = (x0 >= 0.0) ? -rr : rr;
                     sg = -1.0 / (b * (x0 - b));
@@ -205,24 +210,34 @@ __global__ void __launch_bounds__(OT, 1) onestep_kernel(OsArgs o) {
         }
         __syncthreads();
     }
+    // the CTA of the last row has written every entry
+    const double s = os_scale(__ldcg(o.amax));
+    if (s != 1.0) {
+        __syncthreads();
+        for (int j = t; j < n - 1; j += OT) o.alpha[j] /= s;
+    }
 }
 
 // Full skew matrix by rows from the strict lower triangle of A (column-major):
 // F[i * n + j] = A(i, j) below the diagonal, -A(j, i) above.  32 x 32 tiles
-// through shared memory, both sides coalesced.
+// through shared memory, both sides coalesced.  amax: max |A| (os_scale).
 __global__ void __launch_bounds__(256)
-os_full_kernel(int n, const double* __restrict__ A, int lda, double* __restrict__ F, int check, int* status) {
+os_full_kernel(int n, const double* __restrict__ A, int lda, double* __restrict__ F, unsigned long long* amax, int check,
+               int* status) {
     __shared__ double tile[32][33];
     const int bi = blockIdx.x * 32, bj = blockIdx.y * 32;
     if (bi < bj) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     bool bad = false;
+    unsigned long long m = 0;
     for (int jj = ty; jj < 32; jj += 8) {
         const int i = bi + tx, j = bj + jj;
         double v = 0.0;
         if (i < n && j < n && i > j) {
             v = A[(size_t)j * lda + i];
             if (check && !isfinite(v)) bad = true;
+            const unsigned long long b = os_abs_bits(v);
+            m = b > m ? b : m;
         }
         tile[jj][tx] = v;
         // F(j, i) = -A(i, j); the diagonal and the part above it of a diagonal tile come below
@@ -234,6 +249,8 @@ os_full_kernel(int n, const double* __restrict__ A, int lda, double* __restrict_
         const int i = bi + ii, j = bj + tx;
         if (i < n && j < n && i > j) F[(size_t)i * n + j] = tile[tx][ii];
     }
+    m = os_warp_max(m);
+    if (tx == 0 && m > *(volatile unsigned long long*)amax) atomicMax(amax, m);
     if (bad) sk_set_error(status, SKEW_ERR_NONFINITE);
 }
 
@@ -293,11 +310,26 @@ size_t onestep_ws(int n) {
 
 int onestep_vcols(int n) { return n > 2 ? (n - 2 + 63) / 64 * 64 : 64; }
 
-cudaError_t onestep_full(cudaStream_t st, int n, const double* A, int lda, double* F, int check, int* status) {
+namespace {
+// [0] arrivals, [2..3] max |A|
+unsigned* carve_os(Carve& cv, int n, double2** qa) {
+    *qa = cv.take<double2>(2 * (size_t)n);
+    return cv.take<unsigned>(16);
+}
+}  // namespace
+
+int onestep_full(cudaStream_t st, int n, const double* A, int lda, double* F, int check, void* ws, size_t ws_bytes,
+                 int* status) {
+    Carve cv(ws, ws_bytes);
+    double2* qa;
+    unsigned* ctr = carve_os(cv, n, &qa);
+    if (!cv.ok) return SKEW_ERR_WORKSPACE;
+    if (const cudaError_t e = cudaMemsetAsync(ctr, 0, 16 * sizeof(unsigned), st)) return cuda_fail(e);
     const int nb = (n + 31) / 32;
-    os_full_kernel<<<dim3(nb, nb), 256, 0, st>>>(n, A, lda, F, check, status);
+    os_full_kernel<<<dim3(nb, nb), 256, 0, st>>>(n, A, lda, F, reinterpret_cast<unsigned long long*>(ctr + 2), check,
+                                                 status);
     count_launch();
-    return cudaGetLastError();
+    return cuda_ok(cudaGetLastError());
 }
 
 int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, double* alpha, void* ws,
@@ -305,13 +337,12 @@ int onestep_reduce(cudaStream_t st, int n, double* F, double* V, double* tau, do
     if (n < 2) return 0;
     Carve cv(ws, ws_bytes);
     OsArgs o{};
-    o.qa = cv.take<double2>(2 * (size_t)n);
-    o.ctr = cv.take<unsigned>(16);
+    o.ctr = carve_os(cv, n, &o.qa);
     if (!cv.ok) return SKEW_ERR_WORKSPACE;
+    o.amax = reinterpret_cast<const unsigned long long*>(o.ctr + 2);
     const size_t vc = (size_t)onestep_vcols(n);
     if (const cudaError_t e = cudaMemsetAsync(V, 0, sizeof(double) * vc * n, st)) return cuda_fail(e);
     if (const cudaError_t e = cudaMemsetAsync(tau, 0, sizeof(double) * vc, st)) return cuda_fail(e);
-    if (const cudaError_t e = cudaMemsetAsync(o.ctr, 0, sizeof(unsigned), st)) return cuda_fail(e);
     // two rows per CTA and more
     const int G = std::min(device_sms(), (n + 1) / 2);
     if (n > OMAXR * G) return SKEW_ERR_UNSUPPORTED;

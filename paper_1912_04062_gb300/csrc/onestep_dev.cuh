@@ -39,6 +39,33 @@ struct WarpSums {
     }
 };
 
+// The FP64 forms work on s A, s = 1 for max |A| in [2^-400, 2^400] and else the
+// power of two that brings it into [1/2, 1); a column whose tail's squares sum to
+// less than 2^-1000 counts as zero (H = I, below 2^-100 max |A|).  sigma = -1 /
+// (beta u_0) and A x then stay inside the double range: sigma of a plain column
+// leaves it below a norm of 7.5e-155 and above 9.5e153.  The scale is set once a
+// solve: a test in every column, with the column scaled where it needs it, took
+// 60 us of 4.00 ms at n = 500; this takes none that the runs can tell.
+constexpr unsigned TAIL_MIN = 23u << 20;  // 2^-1000
+SK_DEV bool os_tail(double s2) { return (unsigned)__double2hiint(s2) >= TAIL_MIN; }  // NaN too
+// amax: max |A| as the bits of a double, its finite entries
+SK_DEV double os_scale(unsigned long long amax) {
+    const int e = (int)(amax >> 52);
+    return amax == 0 || (unsigned)(e - 623) < 800u ? 1.0 : ldexp(1.0, max(-1000, min(1000, 1022 - e)));
+}
+SK_DEV unsigned long long os_abs_bits(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return b < 0x7ff0000000000000ull ? b : 0ull;
+}
+SK_DEV unsigned long long os_warp_max(unsigned long long m) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_xor_sync(0xffffffffu, m, o);
+        m = w > m ? w : m;
+    }
+    return m;
+}
+
 // The rank-2 update of RC own rows (base, base + stride, ...; matrix rows i0,
 // i0 + G, ...) and their products with x, columns ja + 32 seg + lane + 32 nseg t.
 // coef: sigma u_i and -sigma p_i of the rows.  The row sums of this segment go

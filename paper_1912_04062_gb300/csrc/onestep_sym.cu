@@ -47,7 +47,8 @@ struct F64 {
     static SK_DEV V from(double x) { return x; }
     static SK_DEV double to(V a) { return a; }
     static SK_DEV float lead(V) { return 1.f; }
-    static SK_DEV bool positive(V a) { return a > 0.0; }
+    static SK_DEV bool positive(V a) { return os_tail(a); }
+    static SK_DEV double prescale(unsigned long long amax) { return os_scale(amax); }
     static SK_DEV bool nonneg(V a) { return a >= 0.0; }
     static SK_DEV V root(V a) { return sqrt(a); }
     static SK_DEV V quot(V a, V b) { return a / b; }
@@ -73,6 +74,10 @@ struct DfPair {
     static SK_DEV double to(V a) { return df_to(a); }
     static SK_DEV float lead(V a) { return fabsf(a.x); }
     static SK_DEV bool positive(V a) { return a.x > 0.f; }
+    static SK_DEV double prescale(unsigned long long amax) {
+        const int e = (int)(amax >> 52);
+        return amax == 0 ? 1.0 : ldexp(1.0, max(-1000, min(1000, 1022 - e)));
+    }
     static SK_DEV bool nonneg(V a) { return a.x >= 0.f; }
     static SK_DEV V root(V a) { return df_root(a); }
     static SK_DEV V quot(V a, V b) { return df_quot(a, b); }
@@ -432,8 +437,7 @@ sym_fill_kernel(int n, int T, const double* __restrict__ A, int lda, const unsig
     __shared__ typename Op::V sh[UC][UR + 1];
     const int I = blockIdx.x, J = blockIdx.y;
     if (I < RB * J) return;
-    const int e = (int)(*amax >> 52);
-    const double s = !Op::scaled || *amax == 0 ? 1.0 : ldexp(1.0, max(-1000, min(1000, 1022 - e)));
+    const double s = Op::prescale(*amax);
     if (I == 0 && J == 0 && threadIdx.x == 0) scale[0] = s;
     const int tx = threadIdx.x % UR, ty = threadIdx.x / UR;
     const int i = I * UR + tx;
@@ -488,9 +492,7 @@ int sym_run(cudaStream_t st, int n, const double* A, int lda, double* V, double*
     if (const cudaError_t e = cudaMemsetAsync(w.p, 0, sizeof(double) * T * UC, st)) return cuda_fail(e);
     auto* amax = reinterpret_cast<unsigned long long*>(w.ctr + 2);
     auto* scale = reinterpret_cast<double*>(w.ctr + 4);
-    if (Op::scaled) {
-        if (const int rc = onestep_amax(st, n, A, lda, amax)) return rc;
-    }
+    if (const int rc = onestep_amax(st, n, A, lda, amax)) return rc;
     sym_fill_kernel<Op><<<dim3(UC / Op::UR * T, T), 256, 0, st>>>(n, T, A, lda, amax, static_cast<T8*>(w.tiles), scale, check,
                                                         d_status);
     count_launch();

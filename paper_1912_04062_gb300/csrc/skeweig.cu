@@ -312,11 +312,10 @@ int run_solve(cudaStream_t st, int n, const double* A, int lda, int nev, double*
             count_launch();
             if (p.sym || p.cluster) {
                 // these forms read A themselves
-            } else if (p.refine) {
-                const int rc = onestep_df_full(st, n, A, lda, p.W, check, p.ws_one, p.sz_one, p.status);
-                if (rc) return rc;
-            } else if (const cudaError_t e = onestep_full(st, n, A, lda, p.W, check, p.status)) {
-                return cuda_fail(e);
+            } else if (const int rc =
+                           p.refine ? onestep_df_full(st, n, A, lda, p.W, check, p.ws_one, p.sz_one, p.status)
+                                    : onestep_full(st, n, A, lda, p.W, check, p.ws_one, p.sz_one, p.status)) {
+                return rc;
             }
         }
         mark(1);
