@@ -922,7 +922,9 @@ __device__ __forceinline__ void twist_body(int n, int nev, int kb, int lane, con
         const double n0 = nrm, yr = twist_forward(n, r, half, gam, Y, L, Q, ld, k, live);
         __syncwarp();
         nrm = twist_vector(n, r, yr, true, half, L, Q, ld, k, live, &neg);
-        res = fabs(gam) * sqrt(n0 / nrm);
+        // of an eigenvector the solve grows it by n or so; without a pivot of
+        // size it can grow by any factor, and the residual below says nothing
+        res = nrm <= 1e6 * n * n * n0 ? fabs(gam) * sqrt(n0 / nrm) : INFINITY;
     } else {
         const double dl = gam / nrm;
         if (fabs(dl) < 1e-9) lam += dl;
@@ -934,7 +936,8 @@ __device__ __forceinline__ void twist_body(int n, int nev, int kb, int lane, con
     }
     const double inv = (neg ? -1.0 : 1.0) / sqrt(nrm);
     const double gs = g * sc->down;
-    const bool ok = maxit > 0 && isfinite(inv) && res <= 100.0 * sqrt((double)n) * DBL_EPSILON * gs;
+    // (an overflowed norm has inv = 0)
+    const bool ok = maxit > 0 && inv != 0.0 && isfinite(inv) && res <= 100.0 * sqrt((double)n) * DBL_EPSILON * gs;
     __syncwarp();
     const int h = (n + 1) / 2, lo = half ? h : 0, hi = half ? n : h;
     if (live && ok) {
