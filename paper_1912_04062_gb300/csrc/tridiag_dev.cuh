@@ -836,17 +836,26 @@ __device__ __forceinline__ void clu_body(int n, int nev, int k0, int m, const do
         // modified Gram-Schmidt in index order, normalisation, growth test
         for (int j = 0; j < m; j++) {
             double* qj = Q + k0 + j;
-            for (int p = 0; p < j; p++) {
-                const double* qp = Q + k0 + p;
-                double d = 0.0;
-                for (int i = t; i < n; i += T) d = fma(qp[i * ld], qj[i * ld], d);
-                d = sk_block_sum(d, red);
-                for (int i = t; i < n; i += T) qj[i * ld] = fma(-d, qp[i * ld], qj[i * ld]);
-                __syncthreads();
-            }
+            // a second pass where the first left less than a tenth of the vector:
+            // the rounding of what it took off is then not orthogonal
             double s = 0.0;
-            for (int i = t; i < n; i += T) s = fma(qj[i * ld], qj[i * ld], s);
-            const double nrm = sqrt(sk_block_sum(s, red));
+            for (int pass = 0; pass < 2; pass++) {
+                double off = 0.0;
+                for (int p = 0; p < j; p++) {
+                    const double* qp = Q + k0 + p;
+                    double d = 0.0;
+                    for (int i = t; i < n; i += T) d = fma(qp[i * ld], qj[i * ld], d);
+                    d = sk_block_sum(d, red);
+                    for (int i = t; i < n; i += T) qj[i * ld] = fma(-d, qp[i * ld], qj[i * ld]);
+                    off = fma(d, d, off);
+                    __syncthreads();
+                }
+                s = 0.0;
+                for (int i = t; i < n; i += T) s = fma(qj[i * ld], qj[i * ld], s);
+                s = sk_block_sum(s, red);
+                if (!(s < 1e-2 * off)) break;  // the same in every thread
+            }
+            const double nrm = sqrt(s);
             if (!(nrm > 0.0) || !isfinite(nrm)) {
                 if (t == 0) {
                     s_bad = 1;
