@@ -663,7 +663,7 @@ namespace {
 // Largest order kept in shared memory for a given shared-memory budget per CTA.
 int smem_n_for(size_t budget) {
     int n = 2;
-    while (n < BATCH_SMALL_MAX && smem_reduce(n + 1) <= budget) n++;
+    while (n < BATCH_ONE_CTA && smem_reduce(n + 1) <= budget) n++;
     return n;
 }
 
@@ -672,7 +672,10 @@ int prepare_persistent(int smem_n, int nmax, int count, BatchLaunch* out) {
     const size_t dyn_global = sizeof(double) * (2 * (size_t)nmax + 32);
     const size_t dyn = smem_n >= 2 ? std::max(smem_reduce(smem_n), dyn_global) : dyn_global;
     auto kern = bt_persistent_kernel<MINB>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
+    // a constant: plans of other thresholds, in other threads too, launch the
+    // same kernel with what they need
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_reduce(BATCH_ONE_CTA)) !=
+        cudaSuccess)
         return SKEW_ERR_LAUNCH;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, BT, dyn) != cudaSuccess || occ < 1)
@@ -797,15 +800,16 @@ int batched_prepare(const BatchPlanDev& d, const skew_batched_config& cfg, Batch
     const int dyn_wy = (int)wy_smem(BATCH_MAX, BE);  // a constant: plans of several threads share the kernel
     if (cudaFuncSetAttribute(bt_wy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_wy) != cudaSuccess)
         return SKEW_ERR_LAUNCH;
-    // the shared-memory threshold cannot exceed what the per-SM budget allows
+    // the shared-memory threshold: no more than the per-SM budget allows, nor than
+    // the orders that this kernel gets
     int dev = 0, smem_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     const size_t budget = (size_t)smem_sm / (size_t)cfg.ctas_per_sm - 2048;
-    int smem_n = cfg.smem_max_n;
-    if (smem_n >= 2) smem_n = std::min(smem_n, smem_n_for(budget));
     const int small = d.count - d.nlarge, cnt = small > 0 ? small : 1;
     const int nmax = std::min(d.nmax, BATCH_ONE_CTA);
+    int smem_n = small > 0 ? std::min(cfg.smem_max_n, nmax) : 0;
+    if (smem_n >= 2) smem_n = std::min(smem_n, smem_n_for(budget));
     switch (cfg.ctas_per_sm) {
     case 1: return prepare_persistent<1>(smem_n, nmax, cnt, out);
     case 2: return prepare_persistent<2>(smem_n, nmax, cnt, out);

@@ -899,7 +899,7 @@ int skew_batched_plan_tune(skew_batched_plan* p, skew_batched_config* best, int*
         if (best) *best = p->cfg;
         return 0;
     }
-    static const int kSmem[] = {0, 48, 64, 80, 96, 112, 128, 160};
+    static const int kSmem[] = {0, 48, 64, 80, 96};
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess) return SKEW_ERR_CUDA;
     if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -916,7 +916,8 @@ int skew_batched_plan_tune(skew_batched_plan* p, skew_batched_config* best, int*
             const skew_batched_config c{ctas, kSmem[si], {0, 0}};
             BatchLaunch L{};
             if (batched_prepare(p->d, c, &L)) continue;
-            // thresholds the shared-memory budget caps to the same value time the same launch
+            // thresholds capped to the same value (by the shared-memory budget or the
+            // orders of the batch) time the same launch
             if (L.ctas == last_ctas && L.smem_n == last_smem) continue;
             last_ctas = L.ctas;
             last_smem = L.smem_n;
@@ -947,7 +948,7 @@ int skew_batched_plan_tune(skew_batched_plan* p, skew_batched_config* best, int*
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
-    // keep the fastest (its kernel attribute is set again for the launch)
+    // keep the fastest
     if (batched_prepare(p->d, best_cfg, &best_launch)) return SKEW_ERR_LAUNCH;
     p->cfg = best_cfg;
     p->launch = best_launch;
