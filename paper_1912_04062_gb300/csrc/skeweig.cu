@@ -243,9 +243,9 @@ Plan make_plan(int n, int nev, const skew_opts* o, bool vectors) {
     return p;
 }
 
-// Bytes for (n, nev), never less than for a smaller order: the routes differ in
-// what they hold, and a workspace taken for the largest of several orders has
-// to serve the others.
+// Bytes for (n, nev), never less than for a smaller order with as many vectors or
+// as it has: the routes differ in what they hold, and a workspace taken for the
+// largest of several orders has to serve the others.
 size_t plan_bytes(int n, int nev, const skew_opts* o, bool vectors) {
     auto one = [&](int m) {
         Plan p = make_plan(m, m < n && nev > m / 2 ? m / 2 : nev, o, vectors);
@@ -254,8 +254,9 @@ size_t plan_bytes(int n, int nev, const skew_opts* o, bool vectors) {
         return cv.off;
     };
     size_t bytes = one(n);
-    // the last orders of each route
-    for (int m : {CLUSTER_ONE_MAX, SYM_FP64, SYM_REFINE, ONESTEP_VALUES, ONESTEP_PARTIAL, ONESTEP_FP64_VALUES,
+    // the last orders of each route, and the one with nev vectors as its complete
+    // basis (the refinement's buffers)
+    for (int m : {2 * nev, CLUSTER_ONE_MAX, SYM_FP64, SYM_REFINE, ONESTEP_VALUES, ONESTEP_PARTIAL, ONESTEP_FP64_VALUES,
                   ONESTEP_REFINE, ONESTEP_FP64})
         if (m < n) bytes = one(m) > bytes ? one(m) : bytes;
     return bytes + 256;
