@@ -72,6 +72,7 @@ struct RefineScalars {
     double rnorm2;                 // sum |R~_ij|^2 over the E11 block (orthogonality before the update)
     unsigned long long where;      // packed location of the max: i | j << 20 | blk << 40
     unsigned long long umax_bits;  // max |U_ij| of the update (as double bits)
+    unsigned long long cmax_bits;  // max |E| over the pairs that are not separated
     // the iteration's control on the device (no host round trip): once done is
     // set the remaining launches of the loop return at once
     int done;
@@ -323,7 +324,7 @@ __global__ void refine_etilde_kernel(int m, int n, const double* __restrict__ Wg
     const double tau = refine_tau(n, sc);
     const long long ld = n, mm = (long long)m * m;
     // largest |E|^2 (the square root is taken once, after the loop)
-    double emax2 = 0.0, rn2 = 0.0;
+    double emax2 = 0.0, cmax2 = 0.0, rn2 = 0.0;
     unsigned int close = 0;
     unsigned long long wloc = 0;
     // element (i, j), e = j m + i: threads along i, the grid's y along j (no
@@ -369,6 +370,7 @@ __global__ void refine_etilde_kernel(int m, int n, const double* __restrict__ Wg
             if (a > emax2) { emax2 = a; wloc = (unsigned long long)i | ((unsigned long long)j << 20); }
         } else {
             E11 = cscale(R, 0.5);
+            cmax2 = fmax(cmax2, E11.r * E11.r + E11.i * E11.i);
             if (i != j && !same) close++;
         }
         const cplx num = {Sf.r - lj * F.r, Sf.i - lj * F.i};
@@ -382,6 +384,7 @@ __global__ void refine_etilde_kernel(int m, int n, const double* __restrict__ Wg
             }
         } else {
             E21 = cscale(F, -0.5);
+            cmax2 = fmax(cmax2, E21.r * E21.r + E21.i * E21.i);
             close++;
         }
         Et[e] = E11.r;
@@ -389,8 +392,9 @@ __global__ void refine_etilde_kernel(int m, int n, const double* __restrict__ Wg
         Et[2 * mm + e] = E21.r;
         Et[3 * mm + e] = E21.i;
     }
-    double emax = sqrt(emax2);
+    double emax = sqrt(emax2), cmax = sqrt(cmax2);
     for (int o = 16; o > 0; o >>= 1) {
+        cmax = fmax(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
         const double oe = __shfl_xor_sync(0xffffffffu, emax, o);
         const unsigned long long ow = __shfl_xor_sync(0xffffffffu, wloc, o);
         if (oe > emax) { emax = oe; wloc = ow; }
@@ -400,6 +404,7 @@ __global__ void refine_etilde_kernel(int m, int n, const double* __restrict__ Wg
     if ((threadIdx.x & 31) == 0) {
         const unsigned long long old = atomicMax(&sc->emax_bits, (unsigned long long)__double_as_longlong(emax));
         if ((unsigned long long)__double_as_longlong(emax) > old) atomicExch(&sc->where, wloc);
+        if (cmax > 0.0) atomicMax(&sc->cmax_bits, (unsigned long long)__double_as_longlong(cmax));
         if (close) atomicAdd(&sc->nclose, close);
         atomicAdd(&sc->rnorm2, rn2);
     }
@@ -457,6 +462,7 @@ __global__ void refine_reset_kernel(RefineScalars* sc) {
         sc->rnorm2 = 0.0;
         sc->where = 0ULL;
         sc->umax_bits = 0ULL;
+        sc->cmax_bits = 0ULL;
     }
 }
 
@@ -508,12 +514,19 @@ __global__ void refine_su_kernel(RefineScalars* sc, int it, int sl) {
     }
 }
 
-// End of iteration it: the next iteration would move the vectors by about
-// emax^2, so the loop stops once emax is below 1e-8 (the FP64 level).
+// The next iteration would move the vectors by about the square of this one's
+// largest correction, so the loop stops once that is below 1e-8 (the FP64 level):
+// of the separated pairs (emax), and of the others, whose E = R / 2 or -F / 2 are
+// the steps of a Newton iteration to orthogonality (near a null space F starts
+// at any size).
+__device__ bool refine_converged(const RefineScalars* sc) {
+    return __longlong_as_double((long long)sc->emax_bits) < 1e-8 &&
+           __longlong_as_double((long long)sc->cmax_bits) < 1e-8;
+}
 __global__ void refine_decide_kernel(RefineScalars* sc, int it) {
     if (threadIdx.x != 0 || sc->done) return;
     sc->hist.iterations = it + 1;
-    if (__longlong_as_double((long long)sc->emax_bits) < 1e-8) sc->done = 1;
+    if (refine_converged(sc)) sc->done = 1;
 }
 
 // 2-D grid for the m x m element kernels: x over i (256 threads a block), y
@@ -694,9 +707,10 @@ int refine(cudaStream_t st, int n, const double* A, int lda, double* lambda, dou
             if (h.done) break;
             su = h.su;
             su_dev = nullptr;
-            double emax;
+            double emax, cmax;
             std::memcpy(&emax, &h.emax_bits, sizeof(double));
-            last = emax < 1e-8;  // the device's stop rule (refine_decide_kernel)
+            std::memcpy(&cmax, &h.cmax_bits, sizeof(double));
+            last = emax < 1e-8 && cmax < 1e-8;  // the device's stop rule (refine_converged)
         }
         // the product reads M's digit slices, taken before C is written
         rc = ozaki_split(st, n, n, M, 1, ldn, 1.0, 0, w.oz_mr, w.oz_bytes, &omr, skip);

@@ -259,14 +259,19 @@ __global__ void __launch_bounds__(64) bisect_bd_kernel(int n, int nev, const Tri
     if (k < nev) bisect_bd_body<L>(n, k, gt % L, threadIdx.x & 31, sc, lohi, lambda, a2e, b2e);
 }
 
+// null: a single eigenvalue at NULL_TOL g or below counts as a cluster of one.
 __global__ void clu_list_kernel(int nev, const double* __restrict__ lambda, const TriScalars* sc, double ctol_rel,
-                                int2* __restrict__ list, int* __restrict__ count) {
+                                int null, int2* __restrict__ list, int* __restrict__ count) {
     __shared__ int c;
     if (threadIdx.x == 0) c = 0;
     __syncthreads();
     const double ctol = ctol_rel * sc->g;
-    for (int k = threadIdx.x; k + 1 < nev; k += blockDim.x) {
-        if (!starts_cluster(lambda, k, ctol) || starts_cluster(lambda, k + 1, ctol)) continue;
+    for (int k = threadIdx.x; k < nev; k += blockDim.x) {
+        if (!starts_cluster(lambda, k, ctol)) continue;
+        if (k + 1 == nev || starts_cluster(lambda, k + 1, ctol)) {
+            if (null && lambda[k] <= NULL_TOL * sc->g) list[atomicAdd(&c, 1)] = make_int2(k, 1);
+            continue;
+        }
         int k1 = k + 2;
         while (k1 < nev && !starts_cluster(lambda, k1, ctol)) k1++;
         const int at = atomicAdd(&c, 1);  // clusters are independent: their order does not matter
@@ -345,6 +350,7 @@ invit_clu_df_kernel(int n, int nev, const float* __restrict__ alh, const float* 
             clu_mgs(n, ld, Q, k0, m, red, redi);
             continue;
         }
+        const bool pairs = lambda[k0 + m - 1] <= PAIR_TOL * g;  // halves by themselves
         // the cluster's iterations one after another; st (clu_next_state) is
         // the same in every thread
         int st = 0;
@@ -352,7 +358,7 @@ invit_clu_df_kernel(int n, int nev, const float* __restrict__ alh, const float* 
             for (int j = t; j < m; j += T) {
                 const int k = k0 + j;
                 if (it == 0) {
-                    invit_lu_df(n, alh, all_, lambda[k], ptol, v, ld, k);
+                    invit_lu_df(n, alh, all_, lambda[k] <= NULL_TOL * g ? 0.0 : lambda[k], ptol, v, ld, k);
                     invit_start_df(n, Qd, ld, k);
                 }
                 invit_solve_df(n, v, ld, k);
@@ -364,6 +370,40 @@ invit_clu_df_kernel(int n, int nev, const float* __restrict__ alh, const float* 
             __syncthreads();
             for (int j = 0; j < m; j++) {
                 Df* qj = Qd + k0 + j;
+                if (pairs) {
+                    // twice: with one shift the members start nearly parallel
+                    for (int h = 0; h < 2 * j; h++) {
+                        const Df* qp = Qd + k0 + (h < j ? h : h - j);
+                        Df d[2] = {{0.f, 0.f}, {0.f, 0.f}};
+                        for (int i = t; i < n; i += T)  // T is even: a thread's rows are of one half
+                            d[0] = df_add(d[0], df_mul(qp[i * ld], qj[i * ld]));
+                        d[1] = (t & 1) ? d[0] : Df{0.f, 0.f};
+                        if (t & 1) d[0] = {0.f, 0.f};
+                        d[0] = df_block_sum(d[0], rh, rl);
+                        d[1] = df_block_sum(d[1], rh, rl);
+                        const Df md = {-2.f * d[t & 1].h, -2.f * d[t & 1].l};
+                        for (int i = t; i < n; i += T) qj[i * ld] = df_add(qj[i * ld], df_mul(md, qp[i * ld]));
+                        __syncthreads();
+                    }
+                    double s = 0.0;
+                    for (int i = t; i < n; i += T) {
+                        const double y = df_to_double(qj[i * ld]);
+                        s = fma(y, y, s);
+                    }
+                    const double se = sk_block_sum((t & 1) ? 0.0 : s, red), so = sk_block_sum((t & 1) ? s : 0.0, red);
+                    if (!(se > 0.0) || !(so > 0.0) || !isfinite(se + so)) {
+                        if (t == 0) {
+                            s_bad = 1;
+                            s_ff = min(s_ff, j);
+                        }
+                    } else {
+                        const Df f = df_of(1.0 / sqrt(2.0 * ((t & 1) ? so : se)));
+                        for (int i = t; i < n; i += T) qj[i * ld] = df_mul(qj[i * ld], f);
+                        if (t == 0 && !(sqrt(se + so) >= (double)grow)) s_ff = min(s_ff, j);
+                    }
+                    __syncthreads();
+                    continue;
+                }
                 for (int p = 0; p < j; p++) {
                     const Df* qp = Qd + k0 + p;
                     Df d = {0.f, 0.f};
@@ -574,7 +614,7 @@ int tridiag_eig(cudaStream_t st, int n, const double* alpha, int nev, double* la
             }
             twist_kernel<<<(nev + 15) / 16, 32, 0, st>>>(n, nev, w.a2, alpha, lambda, w.sc, ctol, maxit, fp64 ? 1 : 0,
                                                          w.bf, Qi, w.lohi, w.fail);
-            clu_list_kernel<<<1, 1024, 0, st>>>(nev, lambda, w.sc, ctol, w.clist, w.ccount);
+            clu_list_kernel<<<1, 1024, 0, st>>>(nev, lambda, w.sc, ctol, fp64 ? 0 : 1, w.clist, w.ccount);
             count_launch(2);
             const int cgrid = std::max(1, std::min(nev / 2, 2 * sms));
             if (fp64)

@@ -781,6 +781,17 @@ __device__ __forceinline__ void clu_mgs(int n, size_t ld, double* Q, int k0, int
     }
 }
 
+// Eigenvalues near 0 before a refinement.  It works on the basis [Z, conj(Z)], so
+// the halves of a vector on the even and on the odd rows (real and imaginary part
+// of D q) have to be of norm 2^-1/2, and orthogonal to those of every other
+// vector, each by itself, as they are for an exact lambda > 0.  An eigenvalue
+// known to 2^-43 g leaves a mixture of the vectors of lambda and -lambda where
+// lambda is no larger: below PAIR_TOL g the halves are scaled (and in a cluster
+// orthogonalised) by themselves.  At NULL_TOL g and below, where it may be 0, the
+// shift is 0, with which a solve keeps the halves apart, and the lockstep
+// iteration takes single eigenvalues too.
+constexpr double PAIR_TOL = 0x1p-20, NULL_TOL = 0x1.8p-43;
+
 // Decision after an iteration: state 0 iterating, 1 all members passed (one
 // more iteration), 2 done.  ff = first member that failed the growth test
 // (m if none), bad = a member's norm was zero or not finite.
@@ -909,7 +920,8 @@ __device__ __forceinline__ void twist_body(int n, int nev, int kb, int lane, con
     const size_t ld = (size_t)nev;
     const bool single = starts_cluster(lambda, k, ctol) && (k + 1 >= nev || starts_cluster(lambda, k + 1, ctol));
     const double tight = TIGHT * g;
-    const bool live = kk < nev && (single || (starts_cluster(lambda, k, tight) &&
+    const bool null = !polish && lambda[k] <= NULL_TOL * g;  // left to the lockstep iteration
+    const bool live = kk < nev && !null && (single || (starts_cluster(lambda, k, tight) &&
                                               (k + 1 >= nev || starts_cluster(lambda, k + 1, tight))));
     if (kk < nev && !half) need[2 * k] = live ? 0.0 : 1.0;
     if (!__any_sync(0xffffffffu, live)) return;
@@ -944,9 +956,25 @@ __device__ __forceinline__ void twist_body(int n, int nev, int kb, int lane, con
         res = fabs(gam) / sqrt(nrm);
     }
     const double inv = (neg ? -1.0 : 1.0) / sqrt(nrm);
+    double inv_e = inv, inv_o = inv;  // of the even and the odd rows
+    const bool pair = !polish && live && lambda[k] <= PAIR_TOL * g;
+    if (__any_sync(0xffffffffu, pair)) {
+        __syncwarp();
+        double mine = 0.0;  // lane half 0 the even rows, 1 the odd ones
+        for (int i = half; i < n; i += 2) {
+            const double z = live ? Q[(size_t)i * ld + k] : 0.0;
+            mine = fma(z, z, mine);
+        }
+        const double other = __shfl_xor_sync(0xffffffffu, mine, 16);
+        if (pair) {
+            inv_e = (neg ? -1.0 : 1.0) / sqrt(2.0 * (half ? other : mine));
+            inv_o = (neg ? -1.0 : 1.0) / sqrt(2.0 * (half ? mine : other));
+        }
+    }
     const double gs = g * sc->down;
     // (an overflowed norm has inv = 0)
-    const bool ok = maxit > 0 && inv != 0.0 && isfinite(inv) && res <= 100.0 * sqrt((double)n) * DBL_EPSILON * gs;
+    const bool ok = maxit > 0 && inv != 0.0 && isfinite(inv_e) && isfinite(inv_o) &&
+                    res <= 100.0 * sqrt((double)n) * DBL_EPSILON * gs;
     __syncwarp();
     const int h = (n + 1) / 2, lo = half ? h : 0, hi = half ? n : h;
     if (live && ok) {
@@ -957,7 +985,7 @@ __device__ __forceinline__ void twist_body(int n, int nev, int kb, int lane, con
                 if (i0 + u < hi) z[u] = Q[(size_t)(i0 + u) * ld + k];
 #pragma unroll
             for (int u = 0; u < TW_IB; u++)
-                if (i0 + u < hi) Q[(size_t)(i0 + u) * ld + k] = z[u] * inv;
+                if (i0 + u < hi) Q[(size_t)(i0 + u) * ld + k] = z[u] * ((i0 + u) & 1 ? inv_o : inv_e);
         }
     }
     if (live && !ok && !half) need[2 * k] = 1.0;
