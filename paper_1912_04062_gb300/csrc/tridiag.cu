@@ -358,7 +358,8 @@ invit_clu_df_kernel(int n, int nev, const float* __restrict__ alh, const float* 
             for (int j = t; j < m; j += T) {
                 const int k = k0 + j;
                 if (it == 0) {
-                    invit_lu_df(n, alh, all_, lambda[k] <= NULL_TOL * g ? 0.0 : lambda[k], ptol, v, ld, k);
+                    const bool null = lambda[k] <= NULL_TOL * g;
+                    invit_lu_df(n, alh, all_, null ? 0.0 : lambda[k], ptol, null ? ptol : 0.f, v, ld, k);
                     invit_start_df(n, Qd, ld, k);
                 }
                 invit_solve_df(n, v, ld, k);
@@ -371,35 +372,41 @@ invit_clu_df_kernel(int n, int nev, const float* __restrict__ alh, const float* 
             for (int j = 0; j < m; j++) {
                 Df* qj = Qd + k0 + j;
                 if (pairs) {
-                    // twice: with one shift the members start nearly parallel
+                    // |even|^2 and |odd|^2 of the vector (T is even: a thread's rows
+                    // are of one half)
+                    auto halves = [&]() -> double2 {
+                        double s = 0.0;
+                        for (int i = t; i < n; i += T) {
+                            const double y = df_to_double(qj[i * ld]);
+                            s = fma(y, y, s);
+                        }
+                        const double e = sk_block_sum((t & 1) ? 0.0 : s, red);
+                        return make_double2(e, sk_block_sum((t & 1) ? s : 0.0, red));
+                    };
+                    const double2 before = halves();
+                    // twice: with one shift the members can start nearly parallel
                     for (int h = 0; h < 2 * j; h++) {
                         const Df* qp = Qd + k0 + (h < j ? h : h - j);
-                        Df d[2] = {{0.f, 0.f}, {0.f, 0.f}};
-                        for (int i = t; i < n; i += T)  // T is even: a thread's rows are of one half
-                            d[0] = df_add(d[0], df_mul(qp[i * ld], qj[i * ld]));
-                        d[1] = (t & 1) ? d[0] : Df{0.f, 0.f};
-                        if (t & 1) d[0] = {0.f, 0.f};
-                        d[0] = df_block_sum(d[0], rh, rl);
-                        d[1] = df_block_sum(d[1], rh, rl);
-                        const Df md = {-2.f * d[t & 1].h, -2.f * d[t & 1].l};
+                        Df d = {0.f, 0.f};
+                        for (int i = t; i < n; i += T) d = df_add(d, df_mul(qp[i * ld], qj[i * ld]));
+                        const Df de = df_block_sum((t & 1) ? Df{0.f, 0.f} : d, rh, rl);
+                        const Df dd = df_block_sum((t & 1) ? d : Df{0.f, 0.f}, rh, rl);
+                        const Df md = (t & 1) ? Df{-2.f * dd.h, -2.f * dd.l} : Df{-2.f * de.h, -2.f * de.l};
                         for (int i = t; i < n; i += T) qj[i * ld] = df_add(qj[i * ld], df_mul(md, qp[i * ld]));
                         __syncthreads();
                     }
-                    double s = 0.0;
-                    for (int i = t; i < n; i += T) {
-                        const double y = df_to_double(qj[i * ld]);
-                        s = fma(y, y, s);
-                    }
-                    const double se = sk_block_sum((t & 1) ? 0.0 : s, red), so = sk_block_sum((t & 1) ? s : 0.0, red);
-                    if (!(se > 0.0) || !(so > 0.0) || !isfinite(se + so)) {
+                    const double2 s = halves();
+                    if (!(s.x > 0.0) || !(s.y > 0.0) || !isfinite(s.x + s.y)) {
                         if (t == 0) {
                             s_bad = 1;
                             s_ff = min(s_ff, j);
                         }
                     } else {
-                        const Df f = df_of(1.0 / sqrt(2.0 * ((t & 1) ? so : se)));
+                        const Df f = df_of(1.0 / sqrt(2.0 * ((t & 1) ? s.y : s.x)));
                         for (int i = t; i < n; i += T) qj[i * ld] = df_mul(qj[i * ld], f);
-                        if (t == 0 && !(sqrt(se + so) >= (double)grow)) s_ff = min(s_ff, j);
+                        // nor may a half be the rounding of what the passes took off
+                        if (t == 0 && (!(sqrt(s.x + s.y) >= (double)grow) || s.x < 1e-20 * before.x || s.y < 1e-20 * before.y))
+                            s_ff = min(s_ff, j);
                     }
                     __syncthreads();
                     continue;

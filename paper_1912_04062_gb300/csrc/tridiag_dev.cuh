@@ -486,14 +486,17 @@ __device__ __forceinline__ InvitDf invit_df_view(const InvitBufs& bf, double* Q)
             reinterpret_cast<Df*>(bf.ml), reinterpret_cast<Df*>(Q), bf.sw};
 }
 
+// drop: couplings below it count as zero (the blocks they leave each have a null
+// vector of their own; couplings at rounding level would grow one past all others).
 __device__ __forceinline__ void invit_lu_df(int n, const float* __restrict__ alh, const float* __restrict__ all_,
-                                            double lam, float ptol, const InvitDf& v, size_t ld, int k) {
+                                            double lam, float ptol, float drop, const InvitDf& v, size_t ld, int k) {
     const Df zero = {0.f, 0.f};
     const Df mlam = df_neg(df_of(lam));
-    Df a0 = mlam, a1 = {alh[0], all_[0]};
+    auto edge = [&](int i) { return fabsf(alh[i]) < drop ? zero : Df{alh[i], all_[i]}; };
+    Df a0 = mlam, a1 = edge(0);
     for (int i = 0; i < n - 1; i++) {
-        const Df l = {alh[i], all_[i]};
-        const Df un = (i + 1 < n - 1) ? Df{alh[i + 1], all_[i + 1]} : zero;
+        const Df l = edge(i);
+        const Df un = (i + 1 < n - 1) ? edge(i + 1) : zero;
         const size_t at = i * ld + k;
         if (fabsf(a0.h) >= fabsf(l.h)) {
             Df piv = a0;
