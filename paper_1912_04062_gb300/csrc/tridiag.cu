@@ -284,7 +284,7 @@ __global__ void clu_list_kernel(int nev, const double* __restrict__ lambda, cons
 __global__ void __launch_bounds__(CLU_T)
 invit_clu_kernel(int n, int nev, const double* __restrict__ alpha, const double* __restrict__ lambda,
                  const TriScalars* sc, int maxit, InvitBufs bf, double* Q, const int2* __restrict__ list,
-                 const int* __restrict__ count, const double* __restrict__ need, int* __restrict__ fail) {
+                 const int* __restrict__ count, double* __restrict__ need, int* __restrict__ fail) {
     const int nc = *count;
     for (int b = blockIdx.x; b < nc; b += gridDim.x) {
         __syncthreads();  // the previous cluster is done with shared memory

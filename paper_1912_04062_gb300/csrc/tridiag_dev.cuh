@@ -139,13 +139,15 @@ struct InvitBufs {
 
 // ---- inverse iteration, one vector (column k of the interleaved buffers) ----
 // LU with partial pivoting of S - lam I (U rows u0, u1, u2; multipliers ml;
-// interchanges sw); pivots below ptol are raised to ptol.
+// interchanges sw); pivots below ptol are raised to ptol, couplings below drop
+// count as zero.
 __device__ __forceinline__ void invit_lu(int n, const double* __restrict__ alpha, double lam, double ptol,
-                                         const InvitBufs& bf, size_t ld, int k) {
-    double a0 = -lam, a1 = alpha[0];
+                                         const InvitBufs& bf, size_t ld, int k, double drop = 0.0) {
+    auto edge = [&](int i) { return fabs(alpha[i]) < drop ? 0.0 : alpha[i]; };
+    double a0 = -lam, a1 = edge(0);
     for (int i = 0; i < n - 1; i++) {
-        const double l = alpha[i], dn = -lam;
-        const double un = (i + 1 < n - 1) ? alpha[i + 1] : 0.0;
+        const double l = edge(i), dn = -lam;
+        const double un = (i + 1 < n - 1) ? edge(i + 1) : 0.0;
         const size_t at = i * ld + k;
         if (fabs(a0) >= fabs(l)) {
             double piv = a0;
@@ -807,9 +809,11 @@ __device__ __forceinline__ int clu_next_state(int st, int ff, int m, int bad, in
     return nst;
 }
 
+constexpr double LOST = 2.0;  // need[2 k] of a member to be started again
+
 // One cluster (k0, m) by the CTA.
 __device__ __forceinline__ void clu_body(int n, int nev, int k0, int m, const double* alpha, const double* lambda,
-                                         double g, int maxit, const InvitBufs& bf, double* Q, const double* need,
+                                         double g, int maxit, const InvitBufs& bf, double* Q, double* need,
                                          int* fail) {
     __shared__ double red[32];
     __shared__ int redi[32];
@@ -836,9 +840,10 @@ __device__ __forceinline__ void clu_body(int n, int nev, int k0, int m, const do
         // the members' solves, one thread each
         for (int j = t; j < m; j += T) {
             const int k = k0 + j;
-            if (it == 0) {
-                invit_lu(n, alpha, lambda[k], ptol, bf, ld, k);
+            if (it == 0 || need[2 * k] == LOST) {
+                invit_lu(n, alpha, lambda[k], ptol, bf, ld, k, it == 0 ? 0.0 : ptol);
                 invit_start(n, Q, ld, k);
+                need[2 * k] = 1.0;
             }
             invit_solve(n, bf, Q, ld, k);
         }
@@ -853,6 +858,7 @@ __device__ __forceinline__ void clu_body(int n, int nev, int k0, int m, const do
             // a second pass where the first left less than a tenth of the vector:
             // the rounding of what it took off is then not orthogonal
             double s = 0.0;
+            bool lost = false;
             for (int pass = 0; pass < 2; pass++) {
                 double off = 0.0;
                 for (int p = 0; p < j; p++) {
@@ -868,6 +874,13 @@ __device__ __forceinline__ void clu_body(int n, int nev, int k0, int m, const do
                 for (int i = t; i < n; i += T) s = fma(qj[i * ld], qj[i * ld], s);
                 s = sk_block_sum(s, red);
                 if (!(s < 1e-2 * off)) break;  // the same in every thread
+                lost = lost || s < 1e-14 * off;
+            }
+            // nothing left but rounding: one direction outgrows the others through
+            // couplings at rounding level, so this member starts again without them
+            if (lost && t == 0) {
+                need[2 * (k0 + j)] = LOST;
+                s_ff = min(s_ff, j);
             }
             const double nrm = sqrt(s);
             if (!(nrm > 0.0) || !isfinite(nrm)) {
