@@ -145,6 +145,8 @@ def select_roofline(kinds, form, n, nev, solves, peaks=None, traffic=None):
             name = "qtrd_slide_kernel (FP32)" if form == "mixed" else "qtrd_smem_kernel<double> (FP64)"
         if k == "panel_qr" and direct:
             name = "onestep_sym_kernel (FP64 direct reduction)"
+        if k == "gemm_f64" and direct:
+            name = "gemm_kernel (FP64 back-transformation by the reflectors)"
         if arith == "tensor":
             fl = kinds[k][1] / solves
             peak, bound = peaks["bf16_tflops_sustained"], "tensor"

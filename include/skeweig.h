@@ -92,8 +92,9 @@ typedef enum {
                                       skew_eig_batched) fail as if the pool had no
                                       memory: SKEW_ERR_NOMEM, nothing launched */
 #define SKEW_FAULT_INVIT_NOCONV 2  /* give inverse iteration zero iterations */
-#define SKEW_FAULT_TINY_WAIT 4     /* the solve's waits between CTAs (panel-QR
-                                      grid barrier, bulge-chase progress flags)
+#define SKEW_FAULT_TINY_WAIT 4     /* the solve's waits between CTAs (grid
+                                      barriers and exchanges of the reductions,
+                                      bulge-chase progress flags)
                                       give up after a few polls: a wait that is
                                       not satisfied at once ends the kernel with
                                       SKEW_ERR_DEVICE_TIMEOUT in the status */
@@ -216,7 +217,7 @@ int skew_eig_host(int n, const double* A, int lda, int nev, double* lambda,
  * skew_batched_config below: unblocked Householder tridiagonalisation, one
  * thread-block cluster or one CTA a matrix, largest first; then bisection,
  * the tridiagonals' eigenvectors and the back-transform of all matrices in one
- * launch each), always in FP64; larger orders run the two-step solve of
+ * launch each), always in FP64; larger orders run the single solve of
  * skew_eig_ex one after another in `opts`' mode.  Not in the paper (it solves one matrix per run).
  * Asynchronous on `stream`.  skew_eig_batched takes its workspace from the
  * library pool (stream-ordered, freed on the stream) and reports no per-matrix
@@ -240,14 +241,15 @@ int skew_eig_batched_ex(int count, const int* n, const double* const* A, const i
  * Batched solve as a plan: about ten launches for the whole batch.
  * Not in the paper (it solves one matrix per run; each matrix here follows
  * Algorithm 1 in its one-step form: unblocked Householder tridiagonalisation,
- * Lemma-1 link, bisection and inverse iteration, D map and back
+ * Lemma-1 link, multisection and twisted factorisations, D map and back
  * transformation, FP64 throughout).
  *
  * skew_batched_config sets the reduction of the orders up to 96: ctas_per_sm
  * (1..4) CTAs of 256 threads per SM take matrices from a device work counter,
  * largest first (larger orders take a thread-block cluster each, whose size the
- * library chooses); orders up to smem_max_n (0..160; capped by the shared memory of ctas_per_sm CTAs per SM)
- * keep the working matrix in shared memory, larger ones in global memory.
+ * library chooses); orders up to smem_max_n (0..160; capped at 96, at the
+ * largest order of the batch and by the shared memory of ctas_per_sm CTAs per
+ * SM) keep the working matrix in shared memory, larger ones in global memory.
  * skew_batched_set_config / get_config hold the process-wide default used by
  * skew_eig_batched(_ex) and by plans created with cfg == NULL (initially
  * ctas_per_sm = 2, smem_max_n = 112).

@@ -27,6 +27,9 @@
 // a Rayleigh-Ritz rotation from its FP64-accurate Gram and projection blocks
 // (after Ogita and Aishima's treatment of clustered eigenvalues, 2019), and
 // the first-order terms coupling it to other columns rotate with it.
+// Eigenvalues at 0 are never separated from their conjugates; their vectors have
+// to come with F near 0 (the tridiagonal solver sees to that), since no correction
+// inside the span of Z and conj(Z) can make one from a real vector.
 #include <cfloat>
 #include <cmath>
 #include <cstring>

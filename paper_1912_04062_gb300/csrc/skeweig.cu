@@ -111,11 +111,16 @@ struct Plan {
 // built for, since the two-step route's Q_trd alone costs as much as its whole
 // back-transformation (n = 8192: 2.01 s against 3.56 s, 4000: 0.28 against 0.71).
 // FP64 values only: the reduction against band reduction and chase (8192: 974
-// against 977 ms, 4000: 134 against 228).  Refined: 8192 0.50 s against 0.75 s,
-// 12288 1.78 against 1.82, 16384 3.98 against 3.61; partial vectors take the FP64
-// form against products of 8 slices, chase and double-float Q_trd (a tenth or a
-// fiftieth of them: 4200 169 against 201 ms, 4600 208 / 226, 5000 274 / 254), as
-// do values only (3600 112 / 126, 4100 153 / 146).
+// against 977 ms, 4000: 134 against 228).  Refined (one box, Bethe-Salpeter inputs,
+// then random ones): 8192 500 to 588 against 734 ms (one or two iterations after
+// the direct reduction, three after the two-step one), 500 / 641; 11500 1484 /
+// 1536, 1229 / 1300; 12288 1755 to 1781 / 1786, 1474 / 1492; 13312 2222 / 2148,
+// 1836 / 2117; 16384 3980 / 3610: the line lies below the orders where two
+// iterations make the two equal.  Partial vectors take the FP64 form against
+// products of 8 slices, chase and double-float Q_trd (a tenth or a fiftieth of
+// them: 4200 169 against 201 ms, 4600 208 / 226, 5000 274 / 254), as do values only
+// (3600 112 / 126, 4100 153 / 146).  FP64 with few vectors (20): 9000 1.34 against
+// 3.04 s, 16384 7.40 / 12.0.
 constexpr int ONESTEP_FP64 = 16384, ONESTEP_FP64_VALUES = 8000, ONESTEP_REFINE = 11500, ONESTEP_PARTIAL = 4750,
               ONESTEP_VALUES = 4000;
 // Orders above which the direct reduction keeps the lower triangle only: FP64

