@@ -111,7 +111,7 @@ struct Plan {
 // built for, since the two-step route's Q_trd alone costs as much as its whole
 // back-transformation (n = 8192: 2.01 s against 3.56 s, 4000: 0.28 against 0.71).
 // FP64 values only: the reduction against band reduction and chase (8192: 974
-// against 977 ms, 4000: 134 against 228).  Refined (one box, Bethe-Salpeter inputs,
+// against 977 ms, 4000: 134 against 228).  Refined (one GB300, Bethe-Salpeter inputs,
 // then random ones): 8192 500 to 588 against 734 ms (one or two iterations after
 // the direct reduction, three after the two-step one), 500 / 641; 11500 1484 /
 // 1536, 1229 / 1300; 12288 1755 to 1781 / 1786, 1474 / 1492; 13312 2222 / 2148,
